@@ -2,15 +2,9 @@
 // decoding): one streaming pass over bf16 vocabulary rows.
 //
 // A row is scanned by one CTA, or split over a thread-block cluster of S CTAs
-// when there are too few rows to fill the GPU.  Each thread keeps a register
-// top-k list ordered by (value desc, id asc) and, for stage 1, an online
-// base-2 log-sum-exp (running max + rescaled sum).  A logit enters a list only
-// if it reaches the warp's threshold: the largest k-th best value over the
-// lanes, below which nothing can be in the row's top k (one lane already holds
-// k values at or above it).  Lists and sums are merged by warp shuffles, then
-// across the warps of the CTA through shared memory, then across the cluster
-// through distributed shared memory by the CTA of rank 0, which writes the
-// row's result.  No global scratch is used.  Two ways to feed the lanes:
+// when there are too few rows to fill the GPU.  Top-k lists are ordered by
+// (value desc, id asc); stage 1 also keeps a base-2 log-sum-exp (lazily raised
+// base + sum).  No global scratch is used.  Two ways to feed the lanes:
 //  - register streaming (stage 1): every thread loads 16-byte vectors (8 bf16
 //    logits) with non-allocating loads, the next vectors loaded while the
 //    current ones are consumed; the log-sum-exp work per logit wants the many
@@ -143,13 +137,6 @@ __device__ __forceinline__ void lse_merge(Lse2& a, float mb2, float s2) {
   a.mb = m;
 }
 
-template <int KT, bool LSE>
-struct Part {
-  float v[KT];
-  int i[KT];
-  float mb, s;
-};
-
 __device__ __forceinline__ float max3f(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -188,61 +175,132 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Order-preserving unsigned keys of floats (both zeros map to one key), for
+// warp maxima by one redux instruction instead of five shuffles.  Key 0 lies
+// below every value's, and stands for a NaN too.
+__device__ __forceinline__ uint32_t order_key(float x) {
+  const uint32_t b = __float_as_uint(x + 0.f);
+  if (x != x) return 0u;
+  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float key_value(uint32_t k) {
+  if (k < 0x007fffffu) return -INFINITY;  // keys below every value's
+  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
+}
+__device__ __forceinline__ float warp_max_key(float v) {
+  return key_value(__reduce_max_sync(0xffffffffu, order_key(v)));
+}
+
 // A lower bound on the warp's k-th best value, the same in every lane: the
 // largest lane-local k-th best (that lane holds k values at or above it) and
 // the k-th largest of the lane maxima (k lanes each hold one value at or
 // above it; a lane that ties the current maximum drops out with it, which can
 // only lower the bound).
 template <int KT>
-__device__ __forceinline__ float warp_kth(const TopK<KT>& tk) {
-  float t = warp_max(tk.v[KT - 1]);
-  float m = tk.v[0];
+__device__ __forceinline__ uint32_t warp_kth_key(const TopK<KT>& tk) {
+  uint32_t t = __reduce_max_sync(0xffffffffu, order_key(tk.v[KT - 1]));
+  uint32_t m = order_key(tk.v[0]);
 #pragma unroll
   for (int k = 0; k < KT; ++k) {
-    const float mk = warp_max(m);
-    if (k == KT - 1) t = fmaxf(t, mk);
-    if (m == mk) m = -INFINITY;
+    const uint32_t mk = __reduce_max_sync(0xffffffffu, m);
+    if (k == KT - 1) t = max(t, mk);
+    if (m == mk) m = 0u;
   }
   return t;
 }
-
-template <int KT, bool LSE>
-__device__ __forceinline__ void consume1(float x, int idx, TopK<KT>& tk, Lse2& ls) {
-  if constexpr (LSE) {
-    if (x > ls.m) {
-      const float nb = x * kLog2e;
-      ls.s *= ex2(ls.mb - nb);
-      ls.m = x;
-      ls.mb = nb;
+// A warp's top-k list, the same in every lane: values (as order keys, 0 =
+// empty) and ids, best first.
+template <int KT>
+struct WarpTop {
+  uint32_t key[KT];
+  int id[KT];
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int k = 0; k < KT; ++k) {
+      key[k] = 0u;
+      id[k] = INT_MAX;
     }
-    if (ls.m != -INFINITY) ls.s += ex2(fmaf(x, kLog2e, -ls.mb));
   }
-  tk.insert(x, idx);
+  // (x, ix) goes in behind every entry at or above it: the caller offers equal
+  // values in id order.
+  __device__ __forceinline__ void insert(uint32_t x, int ix) {
+#pragma unroll
+    for (int k = KT - 1; k > 0; --k) {
+      const bool here = x > key[k], above = x > key[k - 1];
+      key[k] = above ? key[k - 1] : here ? x : key[k];
+      id[k] = above ? id[k - 1] : here ? ix : id[k];
+    }
+    if (x > key[0]) {
+      key[0] = x;
+      id[0] = ix;
+    }
+  }
+  // Takes one candidate per lane (key 0: none), best first, lowest id on ties.
+  __device__ __forceinline__ void offer(uint32_t x, int ix) {
+    while (true) {
+      const uint32_t best = __reduce_max_sync(0xffffffffu, x);
+      if (best <= key[KT - 1]) break;
+      const int i = __reduce_min_sync(0xffffffffu, x == best ? ix : INT_MAX);
+      insert(best, i);
+      if (x == best && ix == i) x = 0u;
+    }
+  }
+};
+
+// The warp's list from the lanes' sorted lists: round k takes the best head
+// (largest value, lowest id on ties), and the lane that held it moves on.
+template <int KT>
+__device__ __forceinline__ void warp_merge(TopK<KT>& tk, WarpTop<KT>& out) {
+#pragma unroll
+  for (int k = 0; k < KT; ++k) {
+    const uint32_t x = tk.i[0] == INT_MAX ? 0u : order_key(tk.v[0]);
+    out.key[k] = __reduce_max_sync(0xffffffffu, x);
+    out.id[k] = __reduce_min_sync(0xffffffffu, x == out.key[k] ? tk.i[0] : INT_MAX);
+    if (x == out.key[k] && tk.i[0] == out.id[k]) {
+#pragma unroll
+      for (int q = 0; q + 1 < KT; ++q) {
+        tk.v[q] = tk.v[q + 1];
+        tk.i[q] = tk.i[q + 1];
+      }
+      tk.v[KT - 1] = -INFINITY;
+      tk.i[KT - 1] = INT_MAX;
+    }
+  }
 }
 
-// Ring-fed variant (used for the target argmax, whose light work per logit
-// leaves the loads in flight as the limit).  grid (S, rows) with cluster
-// (S, 1, 1).  TARGET: rows are (b, j) of a [batch][n_max] tree and only
-// j < n_nodes[b] are scanned.
-template <int KT, bool LSE, bool TARGET, int CW>
-__global__ void __launch_bounds__(CW * 32 + 32, CW == 4 ? 6 : 4)
-vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int n_max,
-                  const int32_t* __restrict__ n_nodes, int32_t* __restrict__ top_ids,
-                  float* __restrict__ top_vals, float* __restrict__ margin,
-                  float* __restrict__ logp1, int* err) {
+// The log-sum-exp of the warp's lanes, in every lane.
+__device__ __forceinline__ void warp_lse(Lse2& ls) {
+  const float m = warp_max_key(ls.mb);
+  float sum = m == -INFINITY ? 0.f : ls.s * ex2(ls.mb - m);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  ls.mb = m;
+  ls.s = sum;
+}
+
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The target argmax (ring-fed: its light work per logit leaves the loads in
+// flight as the limit).  grid (S, rows) with cluster (S, 1, 1).  Rows are
+// (b, j) of a [batch][n_max] tree and only j < n_nodes[b] are scanned.
+__global__ void __launch_bounds__(kCtaThreads, 6)
+vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int n_max, const int32_t* __restrict__ n_nodes,
+                  int32_t* __restrict__ targ, int* err) {
   pdl_begin();
   const int64_t row = blockIdx.y;
   const int S = gridDim.x;
   const int c = blockIdx.x;  // rank within the cluster
   const int tid = threadIdx.x;
-
-  if constexpr (TARGET) {
-    const int b = (int)(row / n_max);
-    const int j = (int)(row % n_max);
-    if (j >= n_nodes[b]) {  // uniform over the cluster: every CTA leaves
-      if (c == 0 && tid == 0) top_ids[row] = -1;
-      return;
-    }
+  const int b = (int)(row / n_max);
+  const int j = (int)(row % n_max);
+  if (j >= n_nodes[b]) {  // uniform over the cluster: every CTA leaves
+    if (c == 0 && tid == 0) targ[row] = -1;
+    return;
   }
 
   const uint16_t* rowp = logits + row * (int64_t)vocab;
@@ -254,13 +312,10 @@ vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int
   const int vb = c * per;
   const int ve = min(nvec, vb + per);
 
-  TopK<KT> tk;
+  TopK<1> tk;
   tk.init();
-  Lse2 ls{-INFINITY, -INFINITY, 0.f};
-
-  if (c == 0 && tid < a0) consume1<KT, LSE>(bf16_lo(rowp[tid]), tid, tk, ls);
-  if (c == S - 1 && tid < vocab - tail0)
-    consume1<KT, LSE>(bf16_lo(rowp[tail0 + tid]), tail0 + tid, tk, ls);
+  if (c == 0 && tid < a0) tk.insert(bf16_lo(rowp[tid]), tid);
+  if (c == S - 1 && tid < vocab - tail0) tk.insert(bf16_lo(rowp[tail0 + tid]), tail0 + tid);
 
   const uint4* vp = reinterpret_cast<const uint4*>(rowp + a0);  // 16-byte aligned
   // The CTA's vectors [vb, ve) stream through a ring of kStages shared-memory
@@ -277,109 +332,58 @@ vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int
   if (tid == 0) {
     for (int st = 0; st < kStages; ++st) {
       tc::mbar_init(smem_u32(&full_bar[st]), 1);
-      tc::mbar_init(smem_u32(&empty_bar[st]), CW);
+      tc::mbar_init(smem_u32(&empty_bar[st]), kWarps);
     }
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
 
-  float thr = warp_kth(tk);
-  float mbw = -INFINITY;
-  uint64_t sacc = f2_pack(0.f, 0.f);  // two lane sums, as one f32x2 pair
-  // The threshold and the log-sum-exp base are warp-wide values that all
-  // lanes take part in (the trip count is uniform over the warp):
-  //  - thr: the k-th best value over the warp's lists.  A logit below it
-  //    cannot be in the row's top k (the warp already holds k values at or
-  //    above it), so lists change only in the rare steps with a logit at or
-  //    above it, after which thr is recomputed.
-  //  - mbw: base-2 exponent base of the lane sums (sum of 2^(x log2e - mbw));
-  //    raised, with the sums rescaled, only when some lane sees a logit more
-  //    than 2^8 above it, so the sums stay below 2^8 per term and the rescale
-  //    is rare and uniform.
+  // thr: the warp's maximum so far.  A logit below it cannot be the row's
+  // argmax, so the lanes' best change only in the rare steps with a logit at
+  // or above it, after which thr is recomputed (the trip count is uniform over
+  // the warp, and all lanes take part).
+  float thr = warp_max(tk.v[0]);
   // One step: kUnroll vectors per lane, r[u] at vector index gi[u] (vb-based);
   // FULL when every lane's vectors are in range, so that no check is needed.
-  auto step = [&](const uint4 (&r)[kUnroll], const int (&gi)[kUnroll], int lim, bool first, auto full_tag) {
+  auto step = [&](const uint4 (&r)[kUnroll], const int (&gi)[kUnroll], bool first, auto full_tag) {
     constexpr bool FULL = decltype(full_tag)::value;
-    uint64_t xp[kUnroll][4];  // (lo, hi) logit pairs of each 32-bit word
+    float lo[kUnroll][4], hi[kUnroll][4];
     float gmv[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const uint32_t w[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
-      float lo[4], hi[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        lo[q] = bf16_lo(w[q]);
-        hi[q] = bf16_hi(w[q]);
-        xp[u][q] = f2_pack(lo[q], hi[q]);
+        lo[u][q] = bf16_lo(w[q]);
+        hi[u][q] = bf16_hi(w[q]);
       }
-      const float g = fmaxf(max3f(lo[0], hi[0], lo[1]), max3f(max3f(hi[1], lo[2], hi[2]), lo[3], hi[3]));
-      gmv[u] = (FULL || gi[u] < lim) ? g : -INFINITY;
+      const float g = fmaxf(max3f(lo[u][0], hi[u][0], lo[u][1]),
+                            max3f(max3f(hi[u][1], lo[u][2], hi[u][2]), lo[u][3], hi[u][3]));
+      gmv[u] = (FULL || gi[u] < nloc) ? g : -INFINITY;
     }
-    if constexpr (LSE) {
-      float gl = gmv[0];
-#pragma unroll
-      for (int u = 1; u < kUnroll; ++u) gl = fmaxf(gl, gmv[u]);
-      if (__any_sync(0xffffffffu, gl * kLog2e > mbw + 8.f)) {
-        const float nb = warp_max(gl) * kLog2e;
-        if (mbw != -INFINITY) {
-          const float sc = ex2(mbw - nb);
-          sacc = f2_mul(sacc, f2_pack(sc, sc));
-        }
-        mbw = nb;
-      }
-      if (mbw != -INFINITY) {
-        const uint64_t l2 = f2_pack(kLog2e, kLog2e), nb2 = f2_pack(-mbw, -mbw);
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          if (FULL || gi[u] < lim) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float a, b;
-              f2_unpack(f2_fma(xp[u][q], l2, nb2), a, b);
-              sacc = f2_add(sacc, f2_pack(ex2(a), ex2(b)));
-            }
-          }
-        }
-      }
-    }
-    if (first) {
-      // first step: the k-th largest of the lanes' maxima of this step is a
-      // valid threshold already (each of those maxima is in its lane's list
-      // after the inserts below, or that lane holds k values above it), so
-      // that a warp does not start by inserting every logit it sees
-      float gl = gmv[0];
-#pragma unroll
-      for (int u = 1; u < kUnroll; ++u) gl = fmaxf(gl, gmv[u]);
-#pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        const float mk = warp_max(gl);
-        if (k == KT - 1) thr = fmaxf(thr, mk);
-        if (gl == mk) gl = -INFINITY;
-      }
-    }
+    // a warp does not start by inserting every logit it sees
+    if (first) thr = fmaxf(thr, warp_max(fmaxf(gmv[0], gmv[1])));
     bool cand = false;
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) cand |= (FULL || gi[u] < lim) && gmv[u] >= thr;
+    for (int u = 0; u < kUnroll; ++u) cand |= (FULL || gi[u] < nloc) && gmv[u] >= thr;
     if (__any_sync(0xffffffffu, cand)) {
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        if ((FULL || gi[u] < lim) && gmv[u] >= thr) {
+        if ((FULL || gi[u] < nloc) && gmv[u] >= thr) {
           const int idx = a0 + ((vb + gi[u]) << 3);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            float a, b;
-            f2_unpack(xp[u][q], a, b);
-            if (a >= thr) tk.insert(a, idx + 2 * q);
-            if (b >= thr) tk.insert(b, idx + 2 * q + 1);
+            if (lo[u][q] >= thr) tk.insert(lo[u][q], idx + 2 * q);
+            if (hi[u][q] >= thr) tk.insert(hi[u][q], idx + 2 * q + 1);
           }
         }
       }
-      thr = warp_kth(tk);
+      thr = warp_max(tk.v[0]);
     }
   };
 
-  if (warp == CW) {
+  if (warp == kWarps) {
     // ---------------------------------------------------------------- producer
     if (lane == 0) {
       int issued = 0;
@@ -404,161 +408,113 @@ vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int
       const bool ok = wait_bounded(smem_u32(&full_bar[st]), (ch / kStages) & 1, abort_flag, err, true);
       if (!__all_sync(0xffffffffu, ok)) break;
       const int cb = ch * kChunkVec;              // chunk's first vector (vb-based)
-      const int lim = nloc;
       const bool full = cb + kChunkVec <= nloc;
       // the warp's two steps of this chunk: vectors warp*32 + lane + u*128,
       // u = 0..3; the stage is freed once the second step's vectors are read
       uint4 r[kUnroll];
       int gi[kUnroll];
-#pragma unroll
-      constexpr int kSteps = kChunkVec / (CW * 32 * kUnroll);  // steps per chunk
+      constexpr int kSteps = kChunkVec / (kThreads * kUnroll);  // steps per chunk
 #pragma unroll
       for (int half = 0; half < kSteps; ++half) {
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
-          const int o = warp * 32 + lane + (half * kUnroll + u) * (CW * 32);
+          const int o = warp * 32 + lane + (half * kUnroll + u) * (kThreads);
           gi[u] = cb + o;
-          if (full || gi[u] < lim) r[u] = ld_shared_v4(smem_u32(&ring[st][o]));
+          if (full || gi[u] < nloc) r[u] = ld_shared_v4(smem_u32(&ring[st][o]));
         }
         if (half == kSteps - 1) {
           __syncwarp();
           if (lane == 0) tc::mbar_arrive(smem_u32(&empty_bar[st]));  // this warp's vectors are in registers
         }
-        if (full) step(r, gi, lim, first && half == 0, std::integral_constant<bool, true>());
-        else step(r, gi, lim, first && half == 0, std::integral_constant<bool, false>());
+        if (full) step(r, gi, first && half == 0, std::integral_constant<bool, true>());
+        else step(r, gi, first && half == 0, std::integral_constant<bool, false>());
       }
       first = false;
     }
   }
-  float sa, sb2;
-  f2_unpack(sacc, sa, sb2);
-  const float s0 = sa, s1 = sb2;
-  if constexpr (LSE) lse_merge(ls, mbw, s0 + s1);
 
-  // ---- warp merge
+  // ---- warp, CTA and (rank 0 reading its peers' results) cluster merge
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    tk.merge_shfl(off);
-    if constexpr (LSE) {
-      const float mb2 = __shfl_xor_sync(0xffffffffu, ls.mb, off);
-      const float s2 = __shfl_xor_sync(0xffffffffu, ls.s, off);
-      lse_merge(ls, mb2, s2);
-    }
-  }
-
-  // ---- CTA merge
-  __shared__ Part<KT, LSE> warp_part[CW];
-  __shared__ Part<KT, LSE> cta_part;
-  if (lane == 0 && warp < CW) {
-#pragma unroll
-    for (int k = 0; k < KT; ++k) {
-      warp_part[warp].v[k] = tk.v[k];
-      warp_part[warp].i[k] = tk.i[k];
-    }
-    warp_part[warp].mb = ls.mb;
-    warp_part[warp].s = ls.s;
+  for (int off = 16; off > 0; off >>= 1) tk.merge_shfl(off);
+  __shared__ float warp_v[kWarps], cta_v;
+  __shared__ int warp_i[kWarps], cta_i;
+  if (lane == 0 && warp < kWarps) {
+    warp_v[warp] = tk.v[0];
+    warp_i[warp] = tk.i[0];
   }
   __syncthreads();
-  if (warp == 0) {
-    tk.init();
-    ls.mb = -INFINITY;
-    ls.s = 0.f;
-    if (lane < CW) {
+  if (tid == 0) {
 #pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        tk.v[k] = warp_part[lane].v[k];
-        tk.i[k] = warp_part[lane].i[k];
-      }
-      ls.mb = warp_part[lane].mb;
-      ls.s = warp_part[lane].s;
-    }
-#pragma unroll
-    for (int off = CW / 2; off > 0; off >>= 1) {
-      tk.merge_shfl(off);
-      if constexpr (LSE) {
-        const float mb2 = __shfl_xor_sync(0xffffffffu, ls.mb, off);
-        const float s2 = __shfl_xor_sync(0xffffffffu, ls.s, off);
-        lse_merge(ls, mb2, s2);
-      }
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        cta_part.v[k] = tk.v[k];
-        cta_part.i[k] = tk.i[k];
-      }
-      cta_part.mb = ls.mb;
-      cta_part.s = ls.s;
-    }
+    for (int w = 1; w < kWarps; ++w) tk.insert(warp_v[w], warp_i[w]);
+    cta_v = tk.v[0];
+    cta_i = tk.i[0];
   }
-
-  // ---- cluster merge (rank 0 reads its peers' results through DSMEM)
   if (S > 1) {
     cg::cluster_group cluster = cg::this_cluster();
     cluster.sync();
     if (c == 0 && tid == 0) {
-      for (int r = 1; r < S; ++r) {
-        const Part<KT, LSE>* pp = cluster.map_shared_rank(&cta_part, r);
-#pragma unroll
-        for (int k = 0; k < KT; ++k) tk.insert(pp->v[k], pp->i[k]);
-        if constexpr (LSE) lse_merge(ls, pp->mb, pp->s);
-      }
+      for (int r = 1; r < S; ++r) tk.insert(*cluster.map_shared_rank(&cta_v, r), *cluster.map_shared_rank(&cta_i, r));
     }
     cluster.sync();
-  } else {
-    __syncthreads();
   }
-
-  if (c == 0 && tid == 0) {
-    if constexpr (TARGET) {
-      top_ids[row] = tk.i[0];
-    } else {
-#pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        if (k < k_out) {
-          top_ids[row * k_out + k] = tk.i[k];
-          top_vals[row * k_out + k] = tk.v[k];
-        }
-      }
-      if (margin) margin[row] = tk.v[0] - tk.v[1];
-      if constexpr (LSE) {
-        if (logp1) {
-          const float lse = (ls.mb + log2f(ls.s)) * kLn2;
-          logp1[row] = tk.v[0] - lse;
-        }
-      }
-    }
-  }
+  if (c == 0 && tid == 0) targ[row] = tk.i[0];
 }
 
 // Register-streaming variant (used for stage 1, whose log-sum-exp work per
 // logit wants many resident warps): every thread streams 16-byte vectors with
 // non-allocating loads, the next vectors loaded while the current ones are
-// consumed.  grid (S, rows) with cluster (S, 1, 1).
-// Vectors per lane per step of the register-streaming scan: three 16-byte
-// loads in flight per lane (70 registers, still one wave of the grid).
+// consumed.  grid (S, rows) with cluster (S, 1, 1), T threads per CTA.
+//
+// What bounds it: at 512 rows x 151936 the stream (30.4 us graph-replayed,
+// 5.1 TB/s; 22.9 us at the copy rate); with few rows the latency of a warp's
+// chain of steps and of the merge.  So the rare part of a step and the merge
+// are kept short: warp maxima are one redux instruction on order keys instead
+// of five shuffles; a warp's threshold is shared with the CTA's other warps,
+// so that fewer logits enter a list; every warp writes its result straight
+// into rank 0's shared memory, one cluster barrier follows, and one warp
+// merges all parts at once (before: a merge per CTA, two barriers, and a
+// serial walk over the peers' shared memory by one thread).  Up to top-4 each
+// lane keeps its own list (several logits enter at once, and the code for the
+// inserts stays small: top-3 of 512 x 151936 30.4 us against 37.3 with one
+// list per warp); above, the warp keeps one list, entered one logit at a
+// time, since a lane's 24 unrolled inserts of an 8-deep list no longer fit
+// the instruction cache (top-6 of 512 x 151936: 65 us against 133).
+// Before these changes and the launch shapes of pick_scan: 512 x 151936 top-3
+// 36.7 us, top-6 306 us, 16 x 128256 12.0 us, 128 x 151936 33.6 us (now 14).
+//
+// Vectors per lane per step: three 16-byte loads in flight per lane (70
+// registers up to top-3, still one wave of the grid).
 constexpr int kUnrollS = 3;
+constexpr int kMaxSplit = 8;  // portable cluster size
 
-template <int KT, bool LSE, bool TARGET>
-__global__ void __launch_bounds__(kThreads)
-vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int n_max,
-                  const int32_t* __restrict__ n_nodes, int32_t* __restrict__ top_ids,
-                  float* __restrict__ top_vals, float* __restrict__ margin,
+template <int KT>
+struct ScanPart {
+  uint32_t key[KT];
+  int id[KT];
+  float mb, s;
+};
+
+__device__ __forceinline__ void lse_add(Lse2& ls, float x) { lse_merge(ls, x * kLog2e, 1.f); }
+
+template <int KT, int T>
+__global__ void __launch_bounds__(T)
+vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
+                  int32_t* __restrict__ top_ids, float* __restrict__ top_vals, float* __restrict__ margin,
                   float* __restrict__ logp1) {
-  pdl_begin();
+  constexpr int W = T / 32;
+  __shared__ ScanPart<KT> part[kMaxSplit * W];  // rank 0's holds every warp of the cluster
+  __shared__ uint32_t thr_s;  // the largest k-th best of the CTA's warps, as an order key
   const int64_t row = blockIdx.y;
   const int S = gridDim.x;
   const int c = blockIdx.x;  // rank within the cluster
   const int tid = threadIdx.x;
-
-  if constexpr (TARGET) {
-    const int b = (int)(row / n_max);
-    const int j = (int)(row % n_max);
-    if (j >= n_nodes[b]) {  // uniform over the cluster: every CTA leaves
-      if (c == 0 && tid == 0) top_ids[row] = -1;
-      return;
-    }
-  }
+  const int lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) thr_s = 0u;
+  __syncthreads();
+  // every CTA of the cluster has started once this barrier completes (waited
+  // for before the first write to rank 0's shared memory)
+  if (S > 1) cluster_arrive();
+  pdl_begin();
 
   const uint16_t* rowp = logits + row * (int64_t)vocab;
   const int mis = (int)((reinterpret_cast<uintptr_t>(rowp) >> 1) & 7);
@@ -569,34 +525,43 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int
   const int vb = c * per;
   const int ve = min(nvec, vb + per);
 
-  TopK<KT> tk;
-  tk.init();
-  Lse2 ls{-INFINITY, -INFINITY, 0.f};
-
-  if (c == 0 && tid < a0) consume1<KT, LSE>(bf16_lo(rowp[tid]), tid, tk, ls);
-  if (c == S - 1 && tid < vocab - tail0)
-    consume1<KT, LSE>(bf16_lo(rowp[tail0 + tid]), tail0 + tid, tk, ls);
-
   const uint4* vp = reinterpret_cast<const uint4*>(rowp + a0);
-  // The trip count is uniform over the warp: the threshold and the log-sum-exp
-  // base are warp-wide values that all lanes take part in.
-  //  - thr: the k-th best value over the warp's lists.  A logit below it
-  //    cannot be in the row's top k (the warp already holds k values at or
-  //    above it), so lists change only in the rare steps with a logit at or
-  //    above it, after which thr is recomputed.
-  //  - mbw: base-2 exponent base of the lane sums s0 + s1 (sum of
-  //    2^(x log2e - mbw)); raised, with the sums rescaled, only when some lane
-  //    sees a logit more than 2^8 above it, so the sums stay below 2^8 per
-  //    term and the rescale is rare and uniform.
-  const int lane = tid & 31;
   const int wb0 = vb + (tid & ~31);
   uint4 r[kUnrollS];
 #pragma unroll
   for (int u = 0; u < kUnrollS; ++u) {
-    const int vi = wb0 + lane + u * kThreads;
+    const int vi = wb0 + lane + u * T;
     if (vi < ve) r[u] = ld_stream(vp + vi);
   }
-  float thr = warp_kth(tk);
+
+  constexpr bool kLaneLists = KT <= 4;
+  TopK<KT> ll;      // lane lists, or
+  WarpTop<KT> tk;   // the warp's list
+  ll.init();
+  tk.init();
+  Lse2 ls{-INFINITY, -INFINITY, 0.f};
+  if (c == 0 && warp == 0 && a0 > 0) {  // the ids before the first 16-byte boundary
+    const float x = lane < a0 ? bf16_lo(rowp[lane]) : 0.f;
+    if (lane < a0) lse_add(ls, x);
+    if constexpr (kLaneLists) {
+      if (lane < a0) ll.insert(x, lane);
+    } else {
+      tk.offer(lane < a0 ? order_key(x) : 0u, lane);
+    }
+  }
+
+  // The trip count is uniform over the warp: the list, the threshold and the
+  // log-sum-exp base are warp-wide values that all lanes take part in.
+  //  - tkey: the least order key that can still enter the list: above the
+  //    warp's own k-th best (an equal one comes later in id order), and at or
+  //    above the largest k-th best of the CTA's warps so far (a warp publishes
+  //    its own after each change, and reads the CTA's best once a step).  So
+  //    lists change only in rare steps.
+  //  - mbw: base-2 exponent base of the lane sums (sum of 2^(x log2e - mbw));
+  //    raised, with the sums rescaled, only when some lane sees a logit more
+  //    than 2^8 above it, so the sums stay below 2^8 per term and the rescale
+  //    is rare and uniform.
+  uint32_t tkey = kLaneLists ? 0u : tk.key[KT - 1] + 1u;
   float mbw = -INFINITY;
   uint64_t sacc = f2_pack(0.f, 0.f);  // two lane sums, as one f32x2 pair
   // one step: kUnrollS vectors per lane; FULL when every lane's vectors are in
@@ -606,7 +571,7 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int
     uint4 nx[kUnrollS];
 #pragma unroll
     for (int u = 0; u < kUnrollS; ++u) {
-      const int vi = wb + lane + (kUnrollS + u) * kThreads;
+      const int vi = wb + lane + (kUnrollS + u) * T;
       if (vi < ve) nx[u] = ld_stream(vp + vi);
     }
     uint64_t xp[kUnrollS][4];  // (lo, hi) logit pairs of each 32-bit word
@@ -622,189 +587,241 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out, int
         xp[u][q] = f2_pack(lo[q], hi[q]);
       }
       const float g = fmaxf(max3f(lo[0], hi[0], lo[1]), max3f(max3f(hi[1], lo[2], hi[2]), lo[3], hi[3]));
-      gmv[u] = (FULL || wb + lane + u * kThreads < ve) ? g : -INFINITY;
+      gmv[u] = (FULL || wb + lane + u * T < ve) ? g : -INFINITY;
     }
-    if constexpr (LSE) {
-      float gl = gmv[0];
+    float gl = gmv[0];
 #pragma unroll
-      for (int u = 1; u < kUnrollS; ++u) gl = fmaxf(gl, gmv[u]);
-      if (__any_sync(0xffffffffu, gl * kLog2e > mbw + 8.f)) {
-        const float nb = warp_max(gl) * kLog2e;
-        if (mbw != -INFINITY) {
-          const float sc = ex2(mbw - nb);
-          sacc = f2_mul(sacc, f2_pack(sc, sc));
-        }
-        mbw = nb;
-      }
+    for (int u = 1; u < kUnrollS; ++u) gl = fmaxf(gl, gmv[u]);
+    if (__any_sync(0xffffffffu, gl * kLog2e > mbw + 8.f)) {
+      const float nb = warp_max_key(gl) * kLog2e;
       if (mbw != -INFINITY) {
-        const uint64_t l2 = f2_pack(kLog2e, kLog2e), nb2 = f2_pack(-mbw, -mbw);
-#pragma unroll
-        for (int u = 0; u < kUnrollS; ++u) {
-          if (FULL || wb + lane + u * kThreads < ve) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float a, b;
-              f2_unpack(f2_fma(xp[u][q], l2, nb2), a, b);
-              sacc = f2_add(sacc, f2_pack(ex2(a), ex2(b)));
-            }
-          }
-        }
+        const float sc = ex2(mbw - nb);
+        sacc = f2_mul(sacc, f2_pack(sc, sc));
       }
+      mbw = nb;
     }
-    if (wb == wb0) {
-      // first step: the k-th largest of the lanes' maxima of this step is a
-      // valid threshold already (each of those maxima is in its lane's list
-      // after the inserts below, or that lane holds k values above it), so
-      // that a warp does not start by inserting every logit it sees
-      float gl = gmv[0];
-#pragma unroll
-      for (int u = 1; u < kUnrollS; ++u) gl = fmaxf(gl, gmv[u]);
-#pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        const float mk = warp_max(gl);
-        if (k == KT - 1) thr = fmaxf(thr, mk);
-        if (gl == mk) gl = -INFINITY;
-      }
-    }
-    bool cand = false;
-#pragma unroll
-    for (int u = 0; u < kUnrollS; ++u) cand |= (FULL || wb + lane + u * kThreads < ve) && gmv[u] >= thr;
-    if (__any_sync(0xffffffffu, cand)) {
+    if (mbw != -INFINITY) {
+      const uint64_t l2 = f2_pack(kLog2e, kLog2e), nb2 = f2_pack(-mbw, -mbw);
 #pragma unroll
       for (int u = 0; u < kUnrollS; ++u) {
-        if ((FULL || wb + lane + u * kThreads < ve) && gmv[u] >= thr) {
-          const int idx = a0 + ((wb + lane + u * kThreads) << 3);
+        if (FULL || wb + lane + u * T < ve) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             float a, b;
-            f2_unpack(xp[u][q], a, b);
-            if (a >= thr) tk.insert(a, idx + 2 * q);
-            if (b >= thr) tk.insert(b, idx + 2 * q + 1);
+            f2_unpack(f2_fma(xp[u][q], l2, nb2), a, b);
+            sacc = f2_add(sacc, f2_pack(ex2(a), ex2(b)));
           }
         }
       }
-      thr = warp_kth(tk);
+    }
+    tkey = max(tkey, *reinterpret_cast<volatile uint32_t*>(&thr_s));
+    if constexpr (kLaneLists) {
+      if (wb == wb0) {
+        // first step: the k-th largest of the lanes' maxima of this step is a
+        // valid threshold already, so that a warp does not start by inserting
+        // every logit it sees
+        float gm = gl;
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+          const uint32_t mk = __reduce_max_sync(0xffffffffu, order_key(gm));
+          if (k == KT - 1) tkey = max(tkey, mk);
+          if (gm == key_value(mk)) gm = -INFINITY;
+        }
+      }
+      const float thr = key_value(tkey);
+      if (__any_sync(0xffffffffu, gl >= thr)) {
+#pragma unroll
+        for (int u = 0; u < kUnrollS; ++u) {
+          if ((FULL || wb + lane + u * T < ve) && gmv[u] >= thr) {
+            const int idx = a0 + ((wb + lane + u * T) << 3);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              float a, b;
+              f2_unpack(xp[u][q], a, b);
+              if (a >= thr) ll.insert(a, idx + 2 * q);
+              if (b >= thr) ll.insert(b, idx + 2 * q + 1);
+            }
+          }
+        }
+        tkey = max(tkey, warp_kth_key(ll));
+        if (lane == 0) atomicMax(&thr_s, tkey);
+      }
+    } else if (__any_sync(0xffffffffu, gl >= key_value(tkey))) {
+      // the step's best logits enter one at a time, lowest id on ties; one
+      // that has entered is blanked out as a NaN, which the maxima pass over
+      uint32_t lk = FULL || wb + lane < ve ? order_key(gl) : 0u;
+      while (true) {
+        const uint32_t best = __reduce_max_sync(0xffffffffu, lk);
+        if (best < tkey) break;
+        int at = INT_MAX;  // this lane's first logit equal to it
+        if (lk == best) {
+          const float v = key_value(best);
+#pragma unroll
+          for (int u = kUnrollS - 1; u >= 0; --u) {
+            if (FULL || wb + lane + u * T < ve) {
+              const uint32_t w[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
+#pragma unroll
+              for (int q = 3; q >= 0; --q) {
+                if (bf16_hi(w[q]) == v) at = u * T * 8 + 2 * q + 1;
+                if (bf16_lo(w[q]) == v) at = u * T * 8 + 2 * q;
+              }
+            }
+          }
+        }
+        const int id0 = a0 + ((wb + lane) << 3);
+        const int id = __reduce_min_sync(0xffffffffu, at == INT_MAX ? INT_MAX : id0 + at);
+        tk.insert(best, id);
+        tkey = max(tkey, tk.key[KT - 1] + 1u);
+        if (at != INT_MAX && id0 + at == id) {
+          float g = -INFINITY;
+          bool left = false;
+#pragma unroll
+          for (int u = 0; u < kUnrollS; ++u) {
+            if (FULL || wb + lane + u * T < ve) {
+              uint32_t w[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                if (at == u * T * 8 + 2 * q) w[q] |= 0x00007fffu;
+                if (at == u * T * 8 + 2 * q + 1) w[q] |= 0x7fff0000u;
+                const float lo = bf16_lo(w[q]), hi = bf16_hi(w[q]);
+                g = fmaxf(g, fmaxf(lo, hi));
+                left |= lo == lo || hi == hi;
+              }
+              r[u] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+          lk = left ? order_key(g) : 0u;
+        }
+      }
+      if (lane == 0) atomicMax(&thr_s, tk.key[KT - 1]);
     }
 #pragma unroll
     for (int u = 0; u < kUnrollS; ++u) r[u] = nx[u];
   };
   int wb = wb0;
-  for (; wb + 31 + (kUnrollS - 1) * kThreads < ve; wb += kUnrollS * kThreads)
-    step(wb, std::integral_constant<bool, true>());
-  for (; wb < ve; wb += kUnrollS * kThreads) step(wb, std::integral_constant<bool, false>());
+  for (; wb + 31 + (kUnrollS - 1) * T < ve; wb += kUnrollS * T) step(wb, std::integral_constant<bool, true>());
+  for (; wb < ve; wb += kUnrollS * T) step(wb, std::integral_constant<bool, false>());
   float sa, sb2;
   f2_unpack(sacc, sa, sb2);
-  const float s0 = sa, s1 = sb2;
-  if constexpr (LSE) lse_merge(ls, mbw, s0 + s1);
-
-  // ---- warp merge
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    tk.merge_shfl(off);
-    if constexpr (LSE) {
-      const float mb2 = __shfl_xor_sync(0xffffffffu, ls.mb, off);
-      const float s2 = __shfl_xor_sync(0xffffffffu, ls.s, off);
-      lse_merge(ls, mb2, s2);
+  lse_merge(ls, mbw, sa + sb2);
+  if (c == S - 1 && warp == W - 1 && tail0 < vocab) {  // the ids after the last 16-byte boundary
+    const int i = tail0 + lane;
+    const float x = i < vocab ? bf16_lo(rowp[i]) : 0.f;
+    if (i < vocab) lse_add(ls, x);
+    if constexpr (kLaneLists) {
+      if (i < vocab) ll.insert(x, i);
+    } else {
+      tk.offer(i < vocab ? order_key(x) : 0u, i);
     }
   }
+  if constexpr (kLaneLists) warp_merge(ll, tk);
 
-  // ---- CTA merge
-  __shared__ Part<KT, LSE> warp_part[kWarps];
-  __shared__ Part<KT, LSE> cta_part;
-  const int warp = tid >> 5;
+  // ---- every warp's result goes to rank 0's shared memory
+  warp_lse(ls);
+  if (S > 1) cluster_wait();  // rank 0 has started
   if (lane == 0) {
+    ScanPart<KT>* pp = &part[c * W + warp];
+    if (S > 1) pp = cg::this_cluster().map_shared_rank(pp, 0);
 #pragma unroll
     for (int k = 0; k < KT; ++k) {
-      warp_part[warp].v[k] = tk.v[k];
-      warp_part[warp].i[k] = tk.i[k];
+      pp->key[k] = tk.key[k];
+      pp->id[k] = tk.id[k];
     }
-    warp_part[warp].mb = ls.mb;
-    warp_part[warp].s = ls.s;
+    pp->mb = ls.mb;
+    pp->s = ls.s;
   }
-  __syncthreads();
-  if (warp == 0) {
-    tk.init();
-    ls.mb = -INFINITY;
-    ls.s = 0.f;
-    if (lane < kWarps) {
-#pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        tk.v[k] = warp_part[lane].v[k];
-        tk.i[k] = warp_part[lane].i[k];
-      }
-      ls.mb = warp_part[lane].mb;
-      ls.s = warp_part[lane].s;
-    }
-#pragma unroll
-    for (int off = kWarps / 2; off > 0; off >>= 1) {
-      tk.merge_shfl(off);
-      if constexpr (LSE) {
-        const float mb2 = __shfl_xor_sync(0xffffffffu, ls.mb, off);
-        const float s2 = __shfl_xor_sync(0xffffffffu, ls.s, off);
-        lse_merge(ls, mb2, s2);
-      }
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        cta_part.v[k] = tk.v[k];
-        cta_part.i[k] = tk.i[k];
-      }
-      cta_part.mb = ls.mb;
-      cta_part.s = ls.s;
-    }
-  }
-
-  // ---- cluster merge (rank 0 reads its peers' results through DSMEM)
+  __syncwarp();
   if (S > 1) {
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();
-    if (c == 0 && tid == 0) {
-      for (int r = 1; r < S; ++r) {
-        const Part<KT, LSE>* pp = cluster.map_shared_rank(&cta_part, r);
-#pragma unroll
-        for (int k = 0; k < KT; ++k) tk.insert(pp->v[k], pp->i[k]);
-        if constexpr (LSE) lse_merge(ls, pp->mb, pp->s);
-      }
-    }
-    cluster.sync();
+    cluster_arrive();
+    cluster_wait();
   } else {
     __syncthreads();
   }
+  if (c != 0 || warp != 0) return;
 
-  if (c == 0 && tid == 0) {
-    if constexpr (TARGET) {
-      top_ids[row] = tk.i[0];
-    } else {
+  // ---- rank 0's first warp merges the S * W parts (the vector ranges of the
+  // warps interleave, so equal values of different parts go by id)
+  ls.mb = -INFINITY;
+  ls.s = 0.f;
+  int head[kMaxSplit * W / 32 > 0 ? kMaxSplit * W / 32 : 1];  // next entry of each of this lane's parts
 #pragma unroll
-      for (int k = 0; k < KT; ++k) {
-        if (k < k_out) {
-          top_ids[row * k_out + k] = tk.i[k];
-          top_vals[row * k_out + k] = tk.v[k];
+  for (int j = 0; j < (int)(sizeof(head) / sizeof(int)); ++j) {
+    head[j] = 0;
+    const int p = lane + 32 * j;
+    if (p < S * W) lse_merge(ls, part[p].mb, part[p].s);
+  }
+  float v0 = 0.f, v1 = 0.f;
+  for (int k = 0; k < k_out; ++k) {
+    uint32_t x = 0u;
+    int ix = INT_MAX, from = -1;
+#pragma unroll
+    for (int j = 0; j < (int)(sizeof(head) / sizeof(int)); ++j) {
+      const int p = lane + 32 * j;
+      if (p < S * W && head[j] < KT) {
+        const uint32_t y = part[p].key[head[j]];
+        const int iy = part[p].id[head[j]];
+        if (y > x || (y == x && iy < ix)) {
+          x = y;
+          ix = iy;
+          from = j;
         }
       }
-      if (margin) margin[row] = tk.v[0] - tk.v[1];
-      if constexpr (LSE) {
-        if (logp1) {
-          const float lse = (ls.mb + log2f(ls.s)) * kLn2;
-          logp1[row] = tk.v[0] - lse;
-        }
-      }
+    }
+    const uint32_t best = __reduce_max_sync(0xffffffffu, x);
+    const int id = __reduce_min_sync(0xffffffffu, x == best ? ix : INT_MAX);
+#pragma unroll
+    for (int j = 0; j < (int)(sizeof(head) / sizeof(int)); ++j)
+      if (from == j && x == best && ix == id) ++head[j];
+    float v = key_value(best);
+    if (v == 0.f) v = bf16_lo(rowp[id]);  // the key does not hold a zero's sign
+    if (k == 0) v0 = v;
+    if (k == 1) v1 = v;
+    if (lane == 0) {
+      top_ids[row * k_out + k] = id;
+      top_vals[row * k_out + k] = v;
+    }
+  }
+  warp_lse(ls);
+  if (lane == 0) {
+    if (margin) margin[row] = v0 - v1;
+    if (logp1) {
+      const float lse = (ls.mb + log2f(ls.s)) * kLn2;
+      logp1[row] = v0 - lse;
     }
   }
 }
 
-// One CTA per row once the rows alone give every SM six CTAs (24 warps, the
-// occupancy the scan needs to hide its load and exponential latencies); else
-// split rows over a cluster of up to 8 CTAs, keeping at least two vectors per
-// thread in each.
-int pick_split_lsu(int64_t rows, int vocab) {
+// Launch shape of the register-streaming scan: as many warps per row as fit one
+// wave of the grid (at 70-80 registers an SM holds 28 warps as 4-warp CTAs and
+// 24 as 8-warp ones), a power of two from 4 to 64, since a row's warps stream
+// its parts side by side: with few rows the bytes in flight are what is short.
+// 8-warp CTAs keep the cluster (<= 8 CTAs) within the portable size from 32
+// warps a row on.  Graph-replayed, us per call, against the rule of at most
+// 8 x 4 warps a row that this one replaced (same kernel, top-3):
+//   16 x 128256   8 CTAs x 8 warps  5.3     (8 x 4: 6.2)
+//   64 x 152000   4 x 8            10.8     (8 x 4: 12.2; 8 x 8, two waves: 13.8)
+//   256 x 151937  4 x 4            18.2     (2 x 8: 26.6; 2 x 4: 22.2)
+//   512 x 151936  2 x 4            30.4     (4 x 4: 34.0; 1 x 4: 37.8)
+//   1024 x 128256 1 x 4            43.2     (2 x 4: 47.7; 1 x 8: 46.0)
+// Each CTA keeps at least one vector per thread.
+struct ScanShape {
+  int split, threads;
+};
+ScanShape pick_scan(int64_t rows, int vocab) {
   const int nvec = vocab / 8;
-  if (rows >= 6LL * num_sms()) return 1;
-  int s = (int)((6LL * num_sms() + rows - 1) / rows);
-  s = max(1, min(s, 8));
-  while (s > 1 && nvec / s < 2 * kThreads) --s;
-  return s;
+  const int64_t slots256 = 24LL * num_sms(), slots128 = 28LL * num_sms();  // warps in one wave
+  int t = 128, warps = 4;
+  if (rows * 32 <= slots256) {
+    t = 256;
+    warps = rows * 64 <= slots256 ? 64 : 32;
+  } else if (rows * 16 <= slots128) {
+    warps = 16;
+  } else if (rows * 8 <= slots128) {
+    warps = 8;
+  }
+  int s = warps * 32 / t;
+  while (s > 1 && nvec / s < t) --s;
+  return {s, t};
 }
 
 // The grid is kept to one wave of at most six CTAs per SM (the occupancy the
@@ -822,31 +839,37 @@ int pick_split_ring(int64_t rows, int vocab, int per_sm) {
   return s;
 }
 
-template <int KT, bool LSE, bool TARGET, bool RING, int CW = 4>
-cudaError_t launch_scan(const uint16_t* logits, int64_t rows, int vocab, int k_out, int n_max,
-                        const int32_t* n_nodes, int32_t* top_ids, float* top_vals, float* margin,
-                        float* logp1, cudaStream_t s) {
-  const int S = RING ? pick_split_ring(rows, vocab, CW == 4 ? 6 : 4) : pick_split_lsu(rows, vocab);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(S, (unsigned)rows, 1);
-  cfg.blockDim = dim3(RING ? CW * 32 + 32 : kThreads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
+// Launch attributes shared by both scans: a cluster of S CTAs per row, and a
+// programmatic dependent launch (see pdl_begin()).
+struct ScanLaunch {
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = S;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see pdl_begin()
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  if constexpr (RING)
-    return cudaLaunchKernelEx(&cfg, vocab_ring_kernel<KT, LSE, TARGET, CW>, logits, vocab, k_out, n_max, n_nodes,
-                              top_ids, top_vals, margin, logp1, device_error_word());
-  else
-    return cudaLaunchKernelEx(&cfg, vocab_scan_kernel<KT, LSE, TARGET>, logits, vocab, k_out, n_max, n_nodes,
-                              top_ids, top_vals, margin, logp1);
+  cudaLaunchConfig_t cfg = {};
+  ScanLaunch(int S, int64_t rows, int threads, cudaStream_t s) {
+    cfg.gridDim = dim3(S, (unsigned)rows, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+template <int KT>
+cudaError_t launch_scan(const uint16_t* logits, int64_t rows, int vocab, int k_out, int32_t* top_ids,
+                        float* top_vals, float* margin, float* logp1, cudaStream_t s) {
+  const ScanShape sh = pick_scan(rows, vocab);
+  ScanLaunch l(sh.split, rows, sh.threads, s);
+  switch (sh.threads) {
+    case 256:
+      return cudaLaunchKernelEx(&l.cfg, vocab_scan_kernel<KT, 256>, logits, vocab, k_out, top_ids, top_vals, margin, logp1);
+    default:
+      return cudaLaunchKernelEx(&l.cfg, vocab_scan_kernel<KT, 128>, logits, vocab, k_out, top_ids, top_vals, margin, logp1);
+  }
 }
 
 }  // namespace
@@ -856,10 +879,12 @@ cudaError_t launch_score(const uint16_t* logits, int64_t rows, int vocab, int to
                          cudaStream_t s) {
   if (rows == 0) return cudaSuccess;
   switch (topk) {
-    case 2: return launch_scan<2, true, false, false>(logits, rows, vocab, topk, 0, nullptr, top_ids, top_vals, margin, logp1, s);
-    case 3: return launch_scan<3, true, false, false>(logits, rows, vocab, topk, 0, nullptr, top_ids, top_vals, margin, logp1, s);
-    case 4: return launch_scan<4, true, false, false>(logits, rows, vocab, topk, 0, nullptr, top_ids, top_vals, margin, logp1, s);
-    default: return launch_scan<8, true, false, false>(logits, rows, vocab, topk, 0, nullptr, top_ids, top_vals, margin, logp1, s);
+    case 2: return launch_scan<2>(logits, rows, vocab, topk, top_ids, top_vals, margin, logp1, s);
+    case 3: return launch_scan<3>(logits, rows, vocab, topk, top_ids, top_vals, margin, logp1, s);
+    case 4: return launch_scan<4>(logits, rows, vocab, topk, top_ids, top_vals, margin, logp1, s);
+    case 5:
+    case 6: return launch_scan<6>(logits, rows, vocab, topk, top_ids, top_vals, margin, logp1, s);
+    default: return launch_scan<8>(logits, rows, vocab, topk, top_ids, top_vals, margin, logp1, s);
   }
 }
 
@@ -867,8 +892,8 @@ cudaError_t launch_target_argmax(const uint16_t* logits, int batch, int n_max, i
                                  const int32_t* n_nodes, int32_t* targ, cudaStream_t s) {
   const int64_t rows = (int64_t)batch * n_max;
   if (rows == 0) return cudaSuccess;
-  return launch_scan<1, false, true, true>(logits, rows, vocab, 1, n_max, n_nodes, targ, nullptr,
-                                     nullptr, nullptr, s);
+  ScanLaunch l(pick_split_ring(rows, vocab, 6), rows, kCtaThreads, s);
+  return cudaLaunchKernelEx(&l.cfg, vocab_ring_kernel, logits, vocab, n_max, n_nodes, targ, device_error_word());
 }
 
 }  // namespace cure

@@ -96,6 +96,34 @@ def test_score_draft_one_cta_per_row(cure, rows, V, k):
     _check_scores(cure, W.to_bf16(x), k, sel)
 
 
+@pytest.mark.parametrize("k", [2, 3, 4, 5, 6, 8])
+@pytest.mark.parametrize("rows,V", [(57, 4099), (58, 30011), (114, 2057), (115, 16385), (266, 4111), (267, 4101),
+                                    (532, 4100), (533, 2050), (3, 2047)])
+def test_score_draft_launch_shapes(cure, rows, V, k):
+    """Row counts on both sides of every line of the scan's launch rule, odd
+    vocabularies (rows start at every misalignment), and the rows that stress
+    the lists: ascending (every logit a new best), descending, constant, a few
+    finite logits, both zeros, a very negative one, and (ids only, its margin
+    is no number) all -inf.  Logits stay within 30: the log-sum-exp is formed
+    as float32 base-2 exponents, whose rounding (half an ulp of 30 log2(e), twice)
+    is then 4e-6, within LOGP_TOL; at 300 it would be 4e-5."""
+    rng = np.random.default_rng(rows + V + k)
+    x = rng.standard_normal((rows, V), dtype=np.float32)
+    x[1::9] = np.linspace(-30.0, 30.0, V, dtype=np.float32)
+    x[2::9] = np.linspace(30.0, -30.0, V, dtype=np.float32)
+    x[min(rows - 1, 3)] = 1.5
+    x[5::9] = -np.inf
+    x[5::9, rng.choice(V, 9, replace=False)] = 2.0
+    x[6::9] = np.where(rng.random(V) < 0.5, -0.0, 0.0)
+    x[7::9, -1] = 30.0
+    x[8::9, 0] = -2.0e38
+    sel = np.unique(np.concatenate([np.arange(min(rows, 10)), rng.choice(rows, size=min(rows, 12), replace=False)]))
+    _check_scores(cure, W.to_bf16(x), k, sel)
+    none = torch.full((rows, V), -math.inf, dtype=torch.bfloat16, device=DEV)
+    ids, _, _, _ = cure.cure_score_draft(none, k)
+    assert torch.equal(ids, torch.arange(k, dtype=torch.int32, device=DEV).expand(rows, k))
+
+
 def test_score_draft_full_long_shape_sampled(cure):
     """batch 64 x block 16 x vocab 128256 with top-2: 1024 rows, one CTA per
     row, the launch the long-context configuration takes; 64 sampled rows."""
