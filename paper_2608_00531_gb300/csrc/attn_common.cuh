@@ -17,6 +17,7 @@ struct AttnArgs {
   const uint64_t* anc;
   int batch, n_max, heads_q, G, W, cap;
   int inplace;     // 1: no tree tensors; node j's K/V rows are cache slot L_b + j
+  int cluster;     // > 0: one unit per cluster of this many CTAs (grid units_max * cluster), no workspace
   int units_max;   // piece counters in the workspace
   int unit_cost;   // fixed cost of a unit in the stream-K split, in 64-key tile times
   float scale_log2;
@@ -46,6 +47,11 @@ constexpr int kAttnUnitCost = CURE_ATTN_UNIT_COST;
 #define CURE_ATTN_MIN_TILES 8
 #endif
 constexpr int kAttnMinTiles = CURE_ATTN_MIN_TILES;
+
+constexpr int kAttnMaxCluster = 16;
+// CTAs per unit (2 .. kAttnMaxCluster) when a cluster per unit is the faster
+// form for `units` units of up to `tiles` tiles, else 0 (stream-K).
+int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged);
 
 // The persistent tcgen05 kernel (writes `out`; merges split units itself).
 cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s);

@@ -73,6 +73,8 @@ cudaError_t launch_tree_attn(const AttnPlan& plan, const uint16_t* q, const uint
   const int64_t tiles_unit = (A.cap + kAttnKeys - 1) / kAttnKeys +
                              (A.inplace ? 0 : (n_max + kAttnKeys - 1) / kAttnKeys);
   const int64_t positions = (int64_t)plan.units_max * (tiles_unit + kAttnUnitCost);
+  A.cluster = attn_cluster_size(plan.units_max, tiles_unit, n_max > kAttnRowsCta / A.G, batch > 1);
+  if (A.cluster > 0) return launch_tree_attn_tc(A, dim3(plan.units_max * A.cluster, 1, 1), s);
   int ctas = std::min(num_sms(), kAttnMaxCtas);
   if (kAttnMinTiles > 0)
     ctas = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, positions / kAttnMinTiles));

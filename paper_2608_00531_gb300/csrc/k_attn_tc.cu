@@ -13,6 +13,11 @@
 // piece, and the CTA that completes the unit's last piece (a per-unit counter,
 // fence + atomic, no waiting) merges the pieces and writes the output.
 //
+// With few units a piece's share would be a few tiles and the merge most of the
+// call, so there each unit has a cluster of CTAs to itself instead (at most one
+// piece per CTA): the pieces' results stay in shared memory and all CTAs of the
+// cluster merge a part of the columns each.
+//
 // Roles (12 warps):
 //   warps 0-3 / 4-7   softmax of M tile 0 / 1: thread t owns row t = TMEM lane t
 //                     and writes its bf16 probabilities back into TMEM
@@ -51,6 +56,7 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "attn_common.cuh"
@@ -250,6 +256,27 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// ---- clusters: barrier, a peer's address of a shared-memory variable, loads from it
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+
 // One unit piece owned by this CTA.
 struct Seg {
   int b, h, rg;    // unit
@@ -267,6 +294,10 @@ struct Seg {
 // cost (its piece start-up, epilogue and merge, in tile times) followed by
 // one position per 64-key tile.  The CTA ranges split the cost positions
 // evenly, so a CTA that starts more units gets fewer tiles.
+//
+// CLUSTER: instead, each unit has a cluster of CTAs to itself, which take equal
+// shares of its tiles, one piece each.
+template <bool CLUSTER>
 struct Sched {
   const int* tiles_start;  // smem [B+1]: first cost position of each sequence's units
   const int* units_start;  // smem [B+1]
@@ -284,6 +315,7 @@ struct Sched {
   // g_end; s.next is the position after it.  s.t0 == s.t1 when the range
   // holds no tile of that unit.
   __device__ Seg at(long long g, long long g_end) const {
+    if constexpr (CLUSTER) return of_cluster(g_end);
     int lo = 0, hi = B;  // largest b with tiles_start[b] <= g
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
@@ -317,12 +349,44 @@ struct Sched {
     s.slot = s.u + o0;
     return s;
   }
+  // The one piece of this CTA: share cluster_rank() of unit `unit`.
+  __device__ Seg of_cluster(long long g_end) const {
+    int lo = 0, hi = B;  // largest b with units_start[b] <= unit
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (units_start[mid] <= unit) lo = mid;
+      else hi = mid;
+    }
+    Seg s;
+    s.b = lo;
+    s.L = max(0, min(cache_len[lo], cap));
+    s.n = max(1, min(n_nodes[lo], n_max));
+    if (inplace && s.L + s.n > cap) s.L = max(0, cap - s.n);
+    s.nct = ((inplace ? s.L + s.n : s.L) + BN - 1) / BN;
+    s.T = inplace ? s.nct : s.nct + (s.n + BN - 1) / BN;
+    const int uib = unit - units_start[lo];
+    s.rg = uib / Hkv;
+    s.h = uib % Hkv;
+    s.u = unit;
+    s.t0 = (int)((long long)rank * s.T / csize);
+    s.t1 = (int)((long long)(rank + 1) * s.T / csize);
+    s.parts = csize;
+    s.part = rank;
+    s.slot = 0;
+    s.next = g_end;
+    return s;
+  }
+  int unit, rank, csize;  // CLUSTER: this cluster's unit, this CTA's rank, the cluster size
 };
 
 // INPLACE: the in-place layout (no tree tensors; node j's rows at cache slot
 // L + j), a template parameter so that the separate-tensor kernel carries
 // none of its tests.
-template <bool INPLACE>
+//
+// CLUSTER: one unit per cluster of CTAs, merged through distributed shared
+// memory, for problems with too few units to fill the GPU (see
+// attn_cluster_size for when).
+template <bool INPLACE, bool CLUSTER>
 __global__ void __launch_bounds__(kThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                     const __grid_constant__ CUtensorMap tm_tk, const __grid_constant__ CUtensorMap tm_tv,
@@ -435,7 +499,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kOffTmemSlot);
 
-  Sched sch;
+  Sched<CLUSTER> sch;
   sch.tiles_start = tiles_start;
   sch.units_start = units_start;
   sch.B = B;
@@ -450,9 +514,16 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   sch.cap = A.cap;
   sch.n_max = A.n_max;
   sch.inplace = INPLACE;
-  const bool takes_part = (int)blockIdx.x < sch.P;
-  const long long g_begin = takes_part ? (long long)blockIdx.x * sch.Ttot / sch.P : 0;
-  const long long g_end = takes_part ? (long long)(blockIdx.x + 1) * sch.Ttot / sch.P : 0;
+  if constexpr (CLUSTER) {
+    sch.csize = A.cluster;
+    sch.unit = (int)blockIdx.x / A.cluster;
+    sch.rank = (int)blockIdx.x % A.cluster;
+  }
+  // CLUSTER: this CTA's log-sum-exps [256 rows], over the first K stages' end
+  float* lse_s = reinterpret_cast<float*>(smem + kOffK + 32 * 2 * BM * 16);
+  const bool takes_part = CLUSTER ? sch.unit < units_start[B] : (int)blockIdx.x < sch.P;
+  const long long g_begin = takes_part && !CLUSTER ? (long long)blockIdx.x * sch.Ttot / sch.P : 0;
+  const long long g_end = !takes_part ? 0 : CLUSTER ? 1 : (long long)(blockIdx.x + 1) * sch.Ttot / sch.P;
   // M tile 1 of a piece is active when its first node is a tree node
   auto active1 = [&](const Seg& s) { return (2 * s.rg + 1) * npb < s.n; };
 
@@ -858,6 +929,31 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         if (ok) tc_fence_after();
       }
       // ---- epilogue of the piece
+      if constexpr (CLUSTER) {
+        // normalised O and log-sum-exp into shared memory, over the K and V
+        // stages once no product of either M tile reads them any more: float4
+        // columns [32][256 rows]; merged below
+        named_sync_softmax();
+        const int prow = m * BM + row;
+        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+        if (act && ok) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t o[32];
+            tmem_ld32(tl + kColO + m * 128 + q * 32, o);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              st_shared_v4(sb + kOffK + ((q * 8 + i) * 2 * BM + prow) * 16,
+                           __float_as_uint(__uint_as_float(o[4 * i]) * inv),
+                           __float_as_uint(__uint_as_float(o[4 * i + 1]) * inv),
+                           __float_as_uint(__uint_as_float(o[4 * i + 2]) * inv),
+                           __float_as_uint(__uint_as_float(o[4 * i + 3]) * inv));
+          }
+          lse_s[prow] = m_run + log2f(l_run);
+        }
+        continue;  // (the one piece)
+      }
       const bool whole = s.t0 == 0 && s.t1 == s.T;
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
       // a piece's partial: fp32 float4 columns [32][256 rows], so that the 32
@@ -1002,6 +1098,63 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         }
       }
     }
+    // a CTA of the cluster without tiles (no copy writes its stages) weighs nothing
+    if (CLUSTER && takes_part) {
+      const Seg s = sch.at(0, 1);
+      if (s.t1 <= s.t0) lse_s[tid] = -INFINITY;
+    }
+  }
+
+  if constexpr (CLUSTER) {
+    // ---------------------------------------------------------------- merge
+    // every CTA of the cluster takes 32 / csize float4 columns of all rows:
+    // O = sum_p w_p O_p with w_p = 2^(lse_p - M) / sum_q 2^(lse_q - M)
+    __syncwarp();
+    cluster_sync();
+    if (takes_part && warp < 8) {
+      const Seg s = sch.at(0, 1);
+      const int row = tid & 127, m = warp >> 2;
+      const int node = (2 * s.rg + m) * npb + row / G, gh = row % G;
+      if (row < npb * G && node < s.n) {
+        const uint32_t lse_a = sb + kOffK + 32 * 2 * BM * 16 + tid * 4;
+        float w[kAttnMaxCluster];  // log-sum-exps, then weights (0: no tile of the unit, no O written)
+        float M = -INFINITY, wsum = 0.f;
+#pragma unroll
+        for (int p = 0; p < kAttnMaxCluster; ++p)
+          w[p] = p < sch.csize ? ld_cluster_f32(map_rank(lse_a, p)) : -INFINITY;
+#pragma unroll
+        for (int p = 0; p < kAttnMaxCluster; ++p) M = fmaxf(M, w[p]);
+#pragma unroll
+        for (int p = 0; p < kAttnMaxCluster; ++p) {
+          w[p] = w[p] == -INFINITY ? 0.f : ex2(w[p] - M);
+          wsum += w[p];
+        }
+        const float winv = 1.f / wsum;
+        const int ncol = 32 / sch.csize;  // 2, 4, 8 or 16
+        for (int c0 = sch.rank * ncol; c0 < (sch.rank + 1) * ncol; c0 += 2) {
+          float acc[8] = {};
+          const uint32_t col = sb + kOffK + (c0 * 2 * BM + tid) * 16;
+#pragma unroll
+          for (int p = 0; p < kAttnMaxCluster; ++p) {
+            if (w[p] > 0.f) {
+              const float4 a = ld_cluster_v4(map_rank(col, p)), b = ld_cluster_v4(map_rank(col, p) + 2 * BM * 16);
+              const float wp = w[p] * winv;
+              acc[0] += wp * a.x; acc[1] += wp * a.y; acc[2] += wp * a.z; acc[3] += wp * a.w;
+              acc[4] += wp * b.x; acc[5] += wp * b.y; acc[6] += wp * b.z; acc[7] += wp * b.w;
+            }
+          }
+          uint4 v;
+          v.x = pack_bf16(acc[0], acc[1]);
+          v.y = pack_bf16(acc[2], acc[3]);
+          v.z = pack_bf16(acc[4], acc[5]);
+          v.w = pack_bf16(acc[6], acc[7]);
+          *reinterpret_cast<uint4*>(A.out + (((int64_t)s.b * A.n_max + node) * A.heads_q + s.h * G + gh) * D +
+                                    c0 * 4) = v;
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync();  // the peers have read this CTA's shared memory
   }
 
   tc_fence_before();
@@ -1085,21 +1238,103 @@ bool make_q_map(CUtensorMap* m, const void* base, uint64_t tokens, int Hkv, int 
 
 }  // namespace
 
-cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
-  static std::atomic<uint64_t> attr_done{0};
+namespace {
+
+using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
+                        const AttnArgs);
+constexpr Kernel kKernels[4] = {tree_attn_tc_kernel<false, false>, tree_attn_tc_kernel<true, false>,
+                                tree_attn_tc_kernel<false, true>, tree_attn_tc_kernel<true, true>};
+
+// Dynamic shared memory and clusters above the portable size, once per device.
+cudaError_t set_attributes() {
+  static std::atomic<uint64_t> done{0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const uint64_t bit = 1ull << (dev & 63);
-  if (!(attr_done.load() & bit)) {
-    e = cudaFuncSetAttribute(tree_attn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSmemBytes);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tree_attn_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmemBytes);
+  if (done.load() & bit) return cudaSuccess;
+  for (Kernel k : kKernels) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    attr_done.fetch_or(bit);
   }
+  done.fetch_or(bit);
+  return cudaSuccess;
+}
+
+cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, dim3 grid, int size) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = size;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Clusters of `size` CTAs of the kernel that the device holds at once (a
+// cluster lies within one GPC, so fewer than SMs / size).
+int max_clusters(int size) {
+  static std::atomic<int> known[64][kAttnMaxCluster + 1];  // 1 + the count; 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = known[dev][size].load();
+  if (n == 0) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = cluster_config(attr, dim3(size), size);
+    if (cudaOccupancyMaxActiveClusters(&n, kKernels[2], &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    known[dev][size].store(++n);
+  }
+  return n - 1;
+}
+
+}  // namespace
+
+// The choice between stream-K and a cluster per unit compares two estimates of
+// the call's time in us, fitted to graph-replayed calls (a CTA's time per
+// 64-key tile: 0.65 with one M tile, 1.0 with two):
+//   stream-K: 16 + 1.5 per piece of a unit (its last piece merges the others'
+//             partials alone, through the workspace) + the CTA's tiles; the
+//             lengths of several sequences average about 3/4 of the longest;
+//   clusters: 11 + a CTA's share of the longest unit's tiles, if all units'
+//             clusters are resident at once; the merge runs on all CTAs of the
+//             unit through distributed shared memory.
+// The tiles are counted from the cache's capacity (the lengths are on the
+// device).  Measured, us per call, stream-K -> the cluster size chosen:
+//   1 sequence x 8 kv heads of 4 query heads, 300 / 4096 / 16384 keys
+//                                                  17.0 / 26.5 / 50.8 -> 9.7 / 15.4 / 34.5 (8)
+//   1 x 8, 65536 keys                              75.9 stays (8: 108)
+//   1 x 4 of 7, 4096 keys, in place                34.4 -> 17.7 (16)
+//   4 x 8 of 4, 1000-4096 keys                     30.0 -> 21.3 (4)
+//   8 x 8 of 8, 1024-4096 keys, two M tiles        38.2 stays (2: 40.9)
+//   16 x 4 of 7, 1024-8192 keys                    50.5 stays (2: 66.9)
+int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
+  if (units < 1 || set_attributes() != cudaSuccess) return 0;
+  const int sms = num_sms();
+  const float tile = two_m_tiles ? 1.0f : 0.65f;  // us
+  const float ctas = std::min<float>((float)sms, (float)units * (tiles + kAttnUnitCost) / kAttnMinTiles);
+  float best = 16.f + 1.5f * ctas / units + tile * (ragged ? 0.75f : 1.f) * tiles * units / ctas;
+  int size = 0;
+  for (int c = 2; c <= kAttnMaxCluster; c *= 2) {
+    const float t = 11.f + tile * tiles / c;
+    if (t < best && units <= max_clusters(c)) {
+      best = t;
+      size = c;
+    }
+  }
+  return size;
+}
+
+cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
+  cudaError_t e = set_attributes();
+  if (e != cudaSuccess) return e;
   const int Hkv = A.kv.heads_kv;
   CUtensorMap mk, mv, mtk, mtv, mq;
   bool ok;
@@ -1124,10 +1359,13 @@ cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
   static std::atomic<uint32_t> launches{0};
   AttnArgs a = A;
   a.tag = launches.fetch_add(1) % ((1u << (32 - kCountBits)) - 1) + 1;
-  e = A.inplace ? launch_pdl(tree_attn_tc_kernel<true>, grid, dim3(kThreads), kSmemBytes, s, mk, mv, mtk,
-                             mtv, mq, a)
-                : launch_pdl(tree_attn_tc_kernel<false>, grid, dim3(kThreads), kSmemBytes, s, mk, mv, mtk,
-                             mtv, mq, a);
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = cluster_config(attr, grid, A.cluster > 0 ? A.cluster : 1);
+  cfg.stream = s;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see pdl_begin()
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
+  e = cudaLaunchKernelEx(&cfg, kKernels[(A.inplace ? 1 : 0) + (A.cluster > 0 ? 2 : 0)], mk, mv, mtk, mtv, mq, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

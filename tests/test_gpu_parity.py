@@ -395,6 +395,32 @@ def test_tree_attn_page_sizes(cure, ps, Hq, Hkv):
     _cmp_attn(got, ref, t)
 
 
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("B,Hq,Hkv,lens", [
+    (1, 4, 1, (3,)),                       # one unit, fewer tiles than the 16 CTAs of its cluster
+    (2, 8, 2, (0, 1100)),                  # 16 CTAs a unit, one sequence with an empty cache
+    (1, 32, 8, (700,)),                    # 8
+    (4, 32, 8, (64, 1, 129, 600)),         # 4, ragged
+    (9, 32, 8, (300, 20, 64, 0, 5, 63, 65, 128, 250)),  # 2 (72 units)
+    (1, 64, 1, (500,)),                    # one sequence in several row groups
+])
+def test_tree_attn_few_units(cure, B, Hq, Hkv, lens, paged, in_place):
+    """Problems small enough for a cluster of CTAs per unit: every cluster
+    size, CTAs without a tile, empty caches, one and two M tiles, row groups."""
+    if in_place:
+        t, q, kc, vc, L, table, npages = _in_place_case(B, 16, 8, Hq, Hkv, list(lens), paged, seed=B + Hq)
+        tk = tv = None
+        got = _run_attn_in_place(cure, t, q, kc, vc, L, table, npages, Hkv)
+    else:
+        t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 16, 8, Hq, Hkv, list(lens), paged, 1.0, 1.0, seed=B + Hq)
+        got = _run_attn(cure, t, q, tk, tv, kc, vc, L, table, npages, Hkv)
+        tk, tv = _f64(tk), _f64(tv)
+    ref = oracle.tree_attn(_f64(q), tk, tv, _f64(kc), _f64(vc), L, t["n_nodes"], t["anc"], 1.0 / math.sqrt(128),
+                           table, 16)
+    _cmp_attn(got, ref, t)
+
+
 def test_tree_attn_workspace_contents_do_not_matter(cure):
     """The split-KV workspace may hold anything on entry (old counters of
     other launches, garbage): results match those of a zeroed workspace, call
@@ -422,6 +448,28 @@ def test_tree_attn_workspace_contents_do_not_matter(cure):
                 # run, which may move a result by a bf16 rounding step
                 assert np.all(np.isfinite(got[b, :n])), (fill, b)
                 assert np.abs(got[b, :n] - ref[b, :n]).max() <= 1e-2, (fill, b)
+
+
+@pytest.mark.parametrize("paged", [False, True])
+def test_tree_attn_split_units_on_garbage_workspace(cure, paged):
+    """96 units, too many for a cluster each: the units cut by the stream-K
+    ranges merge through the workspace, whatever it holds on entry."""
+    lens = [900, 37, 1500, 64, 300, 0, 1100, 700, 129, 2000, 511, 1024]
+    t, q, tk, tv, kc, vc, L, table, npages = _attn_case(12, 16, 8, 32, 8, lens, paged, 1.0, 1.0, seed=9)
+    kv = cure.kv_desc(8, 128, table.shape[1], torch.from_numpy(table).to(DEV), 16, npages) if paged else \
+        cure.kv_desc(8, 128, kc.shape[1])
+    ref = oracle.tree_attn(_f64(q), _f64(tk), _f64(tv), _f64(kc), _f64(vc), L, t["n_nodes"], t["anc"],
+                           1.0 / math.sqrt(128), table, 16)
+    args = (q.to(DEV), tk.to(DEV), tv.to(DEV), kc.to(DEV), vc.to(DEV), kv, torch.from_numpy(L).to(DEV),
+            torch.from_numpy(t["n_nodes"].astype(np.int32)).to(DEV),
+            torch.from_numpy(t["anc"].view(np.int64)).to(DEV), 1.0 / math.sqrt(128))
+    nbytes = cure.cure_tree_attn_workspace_size(12, q.shape[1], 32, kv)
+    g = torch.Generator(device=DEV).manual_seed(2)
+    ws = torch.randint(0, 256, (nbytes,), dtype=torch.uint8, device=DEV, generator=g)
+    for _ in range(3):
+        got = cure.cure_tree_attn(*args, workspace=ws).float().cpu().numpy()
+        assert cure.cure_device_error() == 0
+        _cmp_attn(got, ref, t)
 
 
 def test_tree_attn_wide_tree_two_words(cure):

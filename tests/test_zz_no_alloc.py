@@ -147,3 +147,22 @@ def test_noalloc_in_place_layout(env):
         assert ok, ("oracle", b, err)
         ok, err = _close(got, ref[b, :nb].float().cpu())
         assert ok, ("cure_tree_attn", b, err)
+
+
+def test_noalloc_split_units_in_the_static_scratch(env):
+    """96 units, too many for a cluster each: the split units' partials and
+    counters go through the static scratch, in two calls on different inputs."""
+    lib, cure = env
+    lens = (900, 37, 1500, 64, 300, 0, 1100, 700, 129, 2000, 511, 1024)
+    for call, seed in enumerate((5, 6)):
+        x = _inputs(seed, B=12, Hq=32, Hkv=8, lens=lens)
+        kv = cure.kv_desc(8, 128, x["table"].shape[1], x["table"], 16, x["npages"])
+        out = torch.full_like(x["q"], float("nan"))
+        assert _call_noalloc(lib, x, kv, out) == 0
+        torch.cuda.synchronize()
+        assert cure.cure_device_error() == 0
+        want = torch.from_numpy(_oracle(x))
+        for b in range(x["B"]):
+            nb = int(x["t"]["n_nodes"][b])
+            ok, err = _close(out[b, :nb].float().cpu(), want[b, :nb].float())
+            assert ok, (call, b, err)
