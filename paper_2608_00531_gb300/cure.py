@@ -18,19 +18,22 @@ from ._lib import KVDesc, TreeParams, check
 DEVERR_PAGE, DEVERR_SLOT, DEVERR_NODES = _lib.DEVERR_PAGE, _lib.DEVERR_SLOT, _lib.DEVERR_NODES
 
 
-def _stream(stream) -> C.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    if stream is None:
+        # the raw handle: a Stream object per call costs more than the launch of a small kernel
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
-def _p(t: Optional[torch.Tensor]) -> C.c_void_p:
+def _p(t: Optional[torch.Tensor]) -> Optional[int]:
+    """Address of a tensor for the c_void_p arguments (plain ints, which ctypes converts in C)."""
     if t is None:
-        return C.c_void_p(0)
+        return None
     if not t.is_cuda:
         raise ValueError("libcure takes CUDA tensors")
     if not t.is_contiguous():
         raise ValueError("libcure takes contiguous tensors")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _need(t: torch.Tensor, dtype, name: str) -> None:
@@ -49,7 +52,7 @@ def kv_desc(heads_kv: int, head_dim: int, max_len: int, block_table: Optional[to
     d.num_pages = num_pages
     if block_table is not None:
         _need(block_table, torch.int32, "block_table")
-        d.block_table = _p(block_table).value
+        d.block_table = _p(block_table)
         d._keep = block_table  # keep the table alive with the descriptor
     return d
 
@@ -131,21 +134,53 @@ def cure_tree_attn(q: torch.Tensor, tree_k: Optional[torch.Tensor], tree_v: Opti
 
     tree_k = tree_v = None: the in-place layout, node j's K/V rows at cache
     slot cache_len[b] + j."""
-    for t, nm in ((q, "q"), (tree_k, "tree_k"), (tree_v, "tree_v"), (k_cache, "k_cache"),
-                  (v_cache, "v_cache")):
-        if t is not None or nm not in ("tree_k", "tree_v"):
-            _need(t, torch.bfloat16, nm)
+    _need(q, torch.bfloat16, "q")
+    if tree_k is not None:
+        _need(tree_k, torch.bfloat16, "tree_k")
+    if tree_v is not None:
+        _need(tree_v, torch.bfloat16, "tree_v")
+    _need(k_cache, torch.bfloat16, "k_cache")
+    _need(v_cache, torch.bfloat16, "v_cache")
     B, n_max, Hq, D = q.shape
     if out is None:
         out = torch.empty_like(q)
-    need = cure_tree_attn_workspace_size(B, n_max, Hq, kv)
     if workspace is None:
+        need = cure_tree_attn_workspace_size(B, n_max, Hq, kv)
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
     lib = _lib.load()
     check("cure_tree_attn", lib.cure_tree_attn(
         _p(q), _p(tree_k), _p(tree_v), _p(k_cache), _p(v_cache), C.byref(kv), _p(cache_len),
         _p(n_nodes), _p(anc), B, n_max, Hq, float(scale), _p(out), _p(workspace),
         workspace.numel() * workspace.element_size(), _stream(stream)))
+    return out
+
+
+def cure_tree_attn_layers(q: torch.Tensor, tree_k: torch.Tensor, tree_v: torch.Tensor,
+                          k_caches: Sequence[torch.Tensor], v_caches: Sequence[torch.Tensor], kv: KVDesc,
+                          cache_len: torch.Tensor, n_nodes: torch.Tensor, anc: torch.Tensor, scale: float,
+                          out: torch.Tensor, workspace: torch.Tensor, *, stream=None) -> torch.Tensor:
+    """cure_tree_attn of every layer in turn: q, tree_k, tree_v and out are
+    contiguous [layers][...] tensors, the caches one tensor per layer.  The
+    arguments that the layers share are checked and converted once, and a
+    layer's rows are addressed without making views: at one sequence the host
+    work of a call would otherwise outlast its kernel."""
+    for t, nm in ((q, "q"), (tree_k, "tree_k"), (tree_v, "tree_v"), (out, "out")):
+        _need(t, torch.bfloat16, nm)
+    layers, B, n_max, Hq, _ = q.shape
+    if not (len(k_caches) == len(v_caches) == tree_k.shape[0] == tree_v.shape[0] == out.shape[0] == layers):
+        raise ValueError("cure_tree_attn_layers: one cache and one slice per layer")
+    ptrs = [_p(t) for t in (q, tree_k, tree_v, out)]
+    steps = [t.stride(0) * 2 for t in (q, tree_k, tree_v, out)]  # bf16
+    shared = (C.byref(kv), _p(cache_len), _p(n_nodes), _p(anc), B, n_max, Hq, float(scale))
+    ws, ws_bytes, s = _p(workspace), workspace.numel() * workspace.element_size(), _stream(stream)
+    fn = _lib.load().cure_tree_attn
+    (pq, ptk, ptv, po), (sq, stk, stv, so) = ptrs, steps
+    for l in range(layers):
+        k, v = k_caches[l], v_caches[l]
+        _need(k, torch.bfloat16, "k_cache")
+        _need(v, torch.bfloat16, "v_cache")
+        check("cure_tree_attn", fn(pq + l * sq, ptk + l * stk, ptv + l * stv, _p(k), _p(v), *shared, po + l * so,
+                                   ws, ws_bytes, s))
     return out
 
 
@@ -255,8 +290,8 @@ def cure_resync_kv(k_caches: Sequence[torch.Tensor], v_caches: Sequence[torch.Te
         out = dict(draft_valid_len=torch.empty(B, dtype=torch.int32, device=dev),
                    replay_tokens=torch.empty(B, P, dtype=torch.int32, device=dev),
                    n_replay=torch.empty(B, dtype=torch.int32, device=dev))
-    kp = (C.c_void_p * max(1, layers))(*[_p(t).value for t in k_caches])
-    vp = (C.c_void_p * max(1, layers))(*[_p(t).value for t in v_caches])
+    kp = (C.c_void_p * max(1, layers))(*[_p(t) for t in k_caches])
+    vp = (C.c_void_p * max(1, layers))(*[_p(t) for t in v_caches])
     lib = _lib.load()
     check("cure_resync_kv", lib.cure_resync_kv(
         layers, kp, vp, C.byref(kv), _p(tree_k), _p(tree_v), B, n_max, block,

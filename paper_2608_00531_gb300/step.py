@@ -90,15 +90,19 @@ class RepairVerifyStep:
         tree = cure.cure_build_tree(ids, margin, x.root_tok, x.cache_len, self.tau, self.R,
                                     self.branches, self.depth, x.redraft, self.max_ufp,
                                     out=self.tree, stream=stream)
-        for l in range(self.layers):
-            p = self.layer_map[l]
-            cure.cure_tree_attn(x.q[l], x.tree_k[l], x.tree_v[l], k_caches[p], v_caches[p], self.kv,
-                                x.cache_len, tree["n_nodes"], tree["anc"], self.scale,
-                                out=self.attn_out[l], workspace=self.workspace, stream=stream)
-        acc = cure.cure_accept(tree, self.K, target_logits=x.target_logits, targ=self.targ,
-                               out=self.acc, stream=stream)
         kl = [k_caches[self.layer_map[l]] for l in range(self.layers)]
         vl = [v_caches[self.layer_map[l]] for l in range(self.layers)]
+        if all(isinstance(t, torch.Tensor) and t.is_contiguous() and t.dim() == 5 and t.shape[0] == self.layers
+               for t in (x.q, x.tree_k, x.tree_v)):
+            cure.cure_tree_attn_layers(x.q, x.tree_k, x.tree_v, kl, vl, self.kv, x.cache_len, tree["n_nodes"],
+                                       tree["anc"], self.scale, self.attn_out, self.workspace, stream=stream)
+        else:  # layers apart in memory
+            for l in range(self.layers):
+                cure.cure_tree_attn(x.q[l], x.tree_k[l], x.tree_v[l], kl[l], vl[l], self.kv, x.cache_len,
+                                    tree["n_nodes"], tree["anc"], self.scale, out=self.attn_out[l],
+                                    workspace=self.workspace, stream=stream)
+        acc = cure.cure_accept(tree, self.K, target_logits=x.target_logits, targ=self.targ,
+                               out=self.acc, stream=stream)
         rs = cure.cure_resync_kv(kl, vl, self.kv, x.tree_k, x.tree_v, acc, x.cache_len, self.K,
                                  cache_len_out=self.cache_len_out, out=self.rs, stream=stream)
         return dict(score=self.score, tree=tree, attn=self.attn_out, acc=acc, resync=rs)
