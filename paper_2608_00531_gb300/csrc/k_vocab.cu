@@ -784,10 +784,9 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
   warp_lse(ls);
   if (lane == 0) {
     if (margin) margin[row] = v0 - v1;
-    if (logp1) {
-      const float lse = (ls.mb + log2f(ls.s)) * kLn2;
-      logp1[row] = v0 - lse;
-    }
+    // log p = (v0 log2(e) - mb - log2(s)) ln 2: the difference of the two large
+    // exponents is taken first, in one rounding
+    if (logp1) logp1[row] = (fmaf(v0, kLog2e, -ls.mb) - log2f(ls.s)) * kLn2;
   }
 }
 
