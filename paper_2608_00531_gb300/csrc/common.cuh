@@ -102,11 +102,11 @@ cudaError_t launch_resync(int layers, const LayerPtrs& caches, const cure_kv_des
                           int32_t* draft_valid_len, int32_t* replay_tokens, int32_t* n_replay,
                           int* err, cudaStream_t s);
 
-// Fused LM head + argmax: launch plan for a shape (persistent CTAs, one
-// 128-row M tile each, the vocabulary's 128-id halves split into `groups`
+// Fused LM head + argmax: launch plan for a shape (persistent pairs of CTAs, one
+// tile of nt hidden rows each, the vocabulary's 256-id tiles split into `groups`
 // ranges).
 struct LmPlan {
-  int m_tiles = 0, h_tiles = 0, groups = 0;
+  int nt = 0, n_tiles = 0, v_tiles = 0, groups = 0;
   size_t ws_bytes = 0;  // per-range (max, id) partials: groups * rows * 8 bytes
 };
 LmPlan plan_lm_head(int rows, int vocab);

@@ -4,29 +4,44 @@
 //   logits[r][v] = hidden[r] . w_lm[v],   targ[r] = first argmax_v logits[r][v],
 // so that the rows x vocab logits never reach HBM.
 //
-// The contraction runs on the tcgen05 tensor cores: one persistent CTA per SM
-// owns one 128-row M tile of `hidden` and a contiguous range of the vocabulary
-// in 128-id halves, taken as 256-id (N) tiles and, for an odd count, one
-// 128-id tile at its end; the CTAs that share a vocab range run side by side,
-// so each weight tile is read from HBM about once and served to the other M
-// tiles from L2.
-//   warp 0   producer: TMA loads of the 64-wide K slices of the hidden tile
-//            [128 x 64] and of the weight tile [256 x 64] (128-byte swizzle)
-//            into a 4-stage ring;
-//   warp 1   MMA issuer (one lane): per K slice four M128 N256 K16 bf16
-//            products accumulating in float32 in TMEM; two accumulators of
-//            256 columns alternate between N tiles;
-//   warps 2-5 epilogue: each thread owns one TMEM lane (one row), reads the
-//            finished accumulator 32 columns at a time and keeps the row's
-//            running (max, first id), strictly greater replacing, so the lowest
-//            id wins ties; then frees the accumulator for the tile after next.
-// Each CTA writes one (max, id) per row for its vocab range; a second kernel
-// takes the first maximum over the ranges in vocab order.  Waits are bounded:
-// on expiry a CTA flags CURE_DEVERR_TIMEOUT, drains its copies and products,
-// frees its TMEM and leaves.
+// The contraction runs on the tcgen05 tensor cores in pairs of SMs
+// (cta_group::2): a pair owns one N tile of hidden rows (up to 256 columns of
+// the accumulator) and a contiguous range of the vocabulary, taken 256 ids at a
+// time as the M = 256 operand, 128 per CTA.  The pairs that share a vocab range
+// run side by side, so each weight tile is read from HBM about once and served
+// to the other N tiles from L2.
+//   warp 0   producer (each CTA): TMA loads of the 64-wide K slices of its 128
+//            weight rows and of its half of the hidden tile (128-byte swizzle)
+//            into a ring of up to 12 stages; both CTAs' copies complete on the
+//            first CTA's barrier;
+//   warp 1   MMA issuer (one lane of the first CTA): per K slice four
+//            M256 N<=256 K16 bf16 products accumulating in float32 in both
+//            CTAs' TMEM; two accumulators alternate between vocab tiles;
+//   warps 2-9 epilogue (each CTA): a TMEM lane is a vocab id, a column a hidden
+//            row; the warp takes each column's maximum and its first lane (a
+//            redux and a ballot), and the lane that keeps the column replaces
+//            its running (max, id) when strictly greater, so the lowest id
+//            wins ties.
+// The pair merges its 8 lane quarters through the first CTA's shared memory and
+// writes one (max, id) per row for its vocab range; a second kernel takes the
+// first maximum over the ranges.  Waits are bounded: on expiry a CTA flags
+// CURE_DEVERR_TIMEOUT, drains its copies and products, frees its TMEM and
+// leaves.
+//
+// What bounds it: with one tile of rows the weight's bytes (21 x 4096 x 128256:
+// 160 us, 6.6 TB/s); with several the tensor pipe at the clock that the power
+// limit leaves (817 x 4096 x 151936: 640 us, 448 cycles a K slice of 224
+// columns, the products' own time, at 1.44 GHz).  With hidden rows as the N
+// operand 817 rows pad to 896 columns of four tiles that use every SM, and a
+// few rows to 32 instead of a 128-row operand; pairing halves each SM's share
+// of the hidden tile, so the ring holds 7 to 12 slices.  Before (one SM per 128
+// hidden rows x 256 ids, 4 slices): 192 us and 684 us at these shapes, 28.1
+// instead of 12.3 us for 9 x 1024 x 32000 (its reduction over the ranges was a
+// serial loop per row), 103 instead of 90 for 257 x 2048 x 100001.
 #include <cudaTypedefs.h>
-#include <float.h>
+#include <limits.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
@@ -37,59 +52,119 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128;           // rows per M tile (TMEM lanes)
-constexpr int BN = 256;           // vocab ids per N tile (accumulator columns)
-constexpr int BK = 64;            // K slice: one 128-byte swizzled row
-constexpr int NS = 4;             // ring stages
-constexpr int kThreads = 192;     // 6 warps
+constexpr int BV = 128;            // vocab ids per CTA (TMEM lanes); 256 per pair
+constexpr int BN = 256;            // most hidden rows per tile (accumulator columns)
+constexpr int BK = 64;             // K slice: one 128-byte swizzled row
+constexpr int kMaxStages = 12;
+constexpr int kThreads = 320;      // 10 warps
+constexpr int kEpiWarps = 8;
 constexpr uint32_t kTmemCols = 512;
-constexpr int kABytes = BM * BK * 2;       // 16 KiB
-constexpr int kBBytes = BN * BK * 2;       // 32 KiB
-constexpr int kStage = kABytes + kBBytes;  // 48 KiB
-constexpr int kOffBars = NS * kStage;      // 196608
-enum { B_FULL = 0, B_EMPTY = NS, B_ACCFULL = 2 * NS, B_ACCEMPTY = 2 * NS + 2, B_DRAIN = 2 * NS + 4,
-       kNumBars = 2 * NS + 5 };
-constexpr int kOffTmemSlot = kOffBars + 8 * kNumBars;
+constexpr int kABytes = BV * BK * 2;  // 16 KiB
+enum { B_FULL = 0, B_EMPTY = kMaxStages, B_ACCFULL = 2 * kMaxStages, B_ACCEMPTY = B_ACCFULL + 2,
+       B_DRAIN = B_ACCEMPTY + 2, kNumBars = B_DRAIN + 1 };
+constexpr int kOffBars = 0;
+constexpr int kOffTmemSlot = 8 * kNumBars;
 constexpr int kOffAbort = kOffTmemSlot + 4;
-constexpr int kSmemUsed = kOffAbort + 4;
-constexpr int kSmemBytes = kSmemUsed + 1024;  // room to align the base to 1024 bytes
-static_assert(kSmemBytes <= 232448, "fits the 227 KiB opt-in");
+constexpr int kOffRing = 1024;     // stages start 1024-byte aligned
+constexpr int kSmemMax = 232448 - 1024;  // less the room to align the base
+static_assert(kOffAbort + 4 <= kOffRing, "barriers fit below the ring");
+constexpr uint32_t kKeyNegInf = 0x007fffffu;  // order key of -inf
+
+constexpr int stage_bytes(int nt) { return kABytes + nt / 2 * BK * 2; }
+constexpr int stages_of(int nt) {
+  const int n = (kSmemMax - kOffRing) / stage_bytes(nt);
+  return n < kMaxStages ? n : kMaxStages;
+}
 
 struct LmArgs {
   int M, d, V;
-  int m_tiles, groups, h_tiles;  // M tiles, vocab ranges, 128-id vocab halves
-  float* part_val;   // [groups][M]
-  int32_t* part_idx; // [groups][M]
+  int nt, n_tiles;          // hidden rows per tile, tiles
+  int groups, v_tiles;      // vocab ranges, 256-id vocab tiles
+  int stages;
+  uint32_t* part_key;       // [groups][M] order keys of the maxima
+  int32_t* part_idx;        // [groups][M]
   int* err;
 };
 
+// Order-preserving unsigned key of a float (both zeros map to one key); 0
+// stands for a NaN.
+__device__ __forceinline__ uint32_t order_key(float x) {
+  const uint32_t b = __float_as_uint(x + 0.f);
+  if (x != x) return 0u;
+  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of this shared-memory variable in the pair's first CTA.
+__device__ __forceinline__ uint32_t in_first_cta(uint32_t addr) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+  return r;
+}
+__device__ __forceinline__ void arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// All lanes of the warp wait; the warp proceeds only if every lane succeeded.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err) {
+  const bool ok = wait_bounded(bar, parity, abort_flag, err, true);
+  return __all_sync(0xffffffffu, ok);
+}
+// One lane of the (converged) warp.  The issuing warp runs as a whole and elects
+// the lane inside the asm: the descriptors then stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred el;\n\telect.sync _|el, 0xffffffff;\n\tselp.u32 %0, 1, 0, el;\n\t}\n" : "=r"(p));
+  return p != 0;
+}
+
+// A copy into this CTA that completes on a barrier of either CTA of the pair.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
       " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
 
-// Four M128 N256 K16 products over one 64-wide K slice (descriptors step by
-// 32 bytes, 2 in 16-byte units, inside the 128-byte swizzled rows).
+// Four M256 K16 products of the pair over one 64-wide K slice (descriptors step
+// by 32 bytes, 2 in 16-byte units, inside the 128-byte swizzled rows).
 __device__ __forceinline__ void mma_kslice(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p0, pt;\n\t.reg .b64 a, b;\n\t"
+      "{\n\t.reg .pred p0, pt, el;\n\t.reg .b64 a, b;\n\t"
+      "elect.sync _|el, 0xffffffff;\n\t"
       "setp.ne.b32 p0, %4, 0;\n\t"
       "setp.eq.b32 pt, %4, %4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p0;\n\t"
+      "@el tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p0;\n\t"
       "add.s64 a, %1, 2;\n\tadd.s64 b, %2, 2;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, 4;\n\tadd.s64 b, %2, 4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, 6;\n\tadd.s64 b, %2, 6;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t}\n" ::"r"(d),
+      "@el tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, pt;\n\t}\n" ::"r"(d),
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
       : "memory");
 }
+// Arrive on `bar` in both CTAs once the pair's products issued so far are done.
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred el;\n\telect.sync _|el, 0xffffffff;\n\t"
+      "@el tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}\n" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
 
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_constant__ CUtensorMap mw,
                       const LmArgs A) {
   extern __shared__ uint8_t smem_raw[];
@@ -101,13 +176,15 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffAbort);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffTmemSlot);
 
-  const int m_tile = blockIdx.x % A.m_tiles;
-  const int g = blockIdx.x / A.m_tiles;
-  const int h_lo = (int)((int64_t)g * A.h_tiles / A.groups);
-  const int h_hi = (int)((int64_t)(g + 1) * A.h_tiles / A.groups);
-  const int ntl = (h_hi - h_lo + 1) / 2;  // N tiles: 256 ids, the last one 128 for an odd count
-  auto wide = [&](int t) { return h_hi - h_lo - 2 * t >= 2; };
-  const int KS = A.d / BK;
+  const int rank = (int)cluster_rank();
+  const int pair = (int)blockIdx.x >> 1;
+  const int n0 = (pair % A.n_tiles) * A.nt;  // first hidden row of the tile
+  const int g = pair / A.n_tiles;
+  const int t_lo = (int)((int64_t)g * A.v_tiles / A.groups);
+  const int t_hi = (int)((int64_t)(g + 1) * A.v_tiles / A.groups);
+  const int ntl = t_hi - t_lo;
+  const int KS = A.d / BK, NS = A.stages;
+  const int stage = kABytes + A.nt / 2 * BK * 2;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -116,7 +193,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bar(B_ACCFULL + a), 1);
-      mbar_init(bar(B_ACCEMPTY + a), 4);  // one arrival per epilogue warp
+      mbar_init(bar(B_ACCEMPTY + a), 2 * kEpiWarps);  // one arrival per epilogue warp of the pair
     }
     mbar_init(bar(B_DRAIN), 1);
     *abort_flag = 0;
@@ -126,9 +203,15 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
     tma_prefetch_desc(&mh);
     tma_prefetch_desc(&mw);
   }
-  if (warp == 1) tmem_alloc(sb + kOffTmemSlot, kTmemCols);
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sb + kOffTmemSlot),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // both CTAs' barriers and TMEM are ready
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_begin();
@@ -136,136 +219,195 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
     if (lane == 0) {
-      int it = 0;
+      // ring position: stage s, round parity ph (no division by the stage
+      // count: the issuing lanes' instructions set the pace of a slice)
+      int s = 0, it = 0;
+      uint32_t ph = 0, st = sb + kOffRing;
+      const uint32_t full0 = in_first_cta(bar(B_FULL));
+      const int h0 = n0 + rank * (A.nt / 2);
       bool ok = true;
-      for (int t = 0; t < ntl && ok; ++t) {
-        const int v0 = (h_lo + 2 * t) * 128;
-        for (int k = 0; k < KS; ++k, ++it) {
-          const int s = it % NS;
-          if (it >= NS && !wait_bounded(bar(B_EMPTY + s), ((it / NS) & 1) ^ 1, abort_flag, A.err, true)) {
+      for (int t = t_lo; t < t_hi && ok; ++t) {
+        const int v0 = (2 * t + rank) * BV;
+        for (int k = 0; k < KS; ++k) {
+          // (the first round's wait returns at once: the barrier's phase before)
+          if (!wait_bounded(bar(B_EMPTY + s), ph ^ 1u, abort_flag, A.err, true)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(bar(B_FULL + s), kStage);
-          const uint32_t st = sb + s * kStage;
-          tma_load_2d(st, &mh, bar(B_FULL + s), k * BK, m_tile * BM);
-          // a 128-id tile still loads a whole box; its second half goes unused
-          tma_load_2d(st + kABytes, &mw, bar(B_FULL + s), k * BK, v0);
+          if (rank == 0) mbar_arrive_expect_tx(bar(B_FULL + s), 2 * stage);  // both CTAs' copies
+          tma_load_2d(st, &mw, full0 + 8u * s, k * BK, v0);
+          tma_load_2d(st + kABytes, &mh, full0 + 8u * s, k * BK, h0);
+          ++it;
+          st += stage;
+          if (++s == NS) {
+            s = 0;
+            ph ^= 1u;
+            st = sb + kOffRing;
+          }
         }
       }
       if (!ok) {  // let the copies in flight land before the CTA's smem goes away
-        for (int j = max(0, it - NS); j < it; ++j)
-          wait_bounded(bar(B_FULL + j % NS), (j / NS) & 1, abort_flag, A.err, false);
+        if (rank == 0) {
+          for (int j = max(0, it - NS); j < it; ++j)
+            wait_bounded(bar(B_FULL + j % NS), (j / NS) & 1, abort_flag, A.err, false);
+        } else {  // they complete on the other CTA's barriers: a time far above a copy's
+          const long long t0 = clock64();
+          while (clock64() - t0 < (1 << 20)) {
+          }
+        }
       }
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc_w = idesc_bf16_f32(BM, BN, false);
-      constexpr uint32_t idesc_h = idesc_bf16_f32(BM, BN / 2, false);
-      int it = 0;
+    if (rank == 0) {
+      const uint32_t idesc = idesc_bf16_f32(2 * BV, A.nt, false);
+      int s = 0;
+      uint32_t ph = 0;
+      const uint64_t ad0 = sdesc_sw128(sb + kOffRing, 16, 1024), bd0 = sdesc_sw128(sb + kOffRing + kABytes, 16, 1024);
+      uint32_t off = 0;  // of the stage, in the descriptors' 16-byte units
       bool ok = true;
       for (int t = 0; t < ntl && ok; ++t) {
         const int a = t & 1;
-        if (t >= 2 && !wait_bounded(bar(B_ACCEMPTY + a), ((t >> 1) & 1) ^ 1, abort_flag, A.err, true)) {
+        if (t >= 2 && !wait_warp(bar(B_ACCEMPTY + a), ((t >> 1) & 1) ^ 1, abort_flag, A.err)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t idesc = wide(t) ? idesc_w : idesc_h;
-        for (int k = 0; k < KS; ++k, ++it) {
-          const int s = it % NS;
-          if (!wait_bounded(bar(B_FULL + s), (it / NS) & 1, abort_flag, A.err, true)) {
+        for (int k = 0; k < KS; ++k) {
+          if (!wait_warp(bar(B_FULL + s), ph, abort_flag, A.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t st = sb + s * kStage;
-          mma_kslice(tmem + a * BN, sdesc_sw128(st, 16, 1024), sdesc_sw128(st + kABytes, 16, 1024), idesc,
-                     k > 0 ? 1u : 0u);
-          mma_commit(bar(B_EMPTY + s));
+          mma_kslice(tmem + a * BN, ad0 + off, bd0 + off, idesc, k > 0 ? 1u : 0u);
+          commit_pair(bar(B_EMPTY + s));
+          off += (uint32_t)stage >> 4;
+          if (++s == NS) {
+            s = 0;
+            ph ^= 1u;
+            off = 0;
+          }
         }
-        if (ok) mma_commit(bar(B_ACCFULL + a));
+        if (ok) commit_pair(bar(B_ACCFULL + a));
       }
       // every product issued has completed before TMEM is freed
-      mma_commit(bar(B_DRAIN));
+      if (elect_one())
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar(B_DRAIN))
+                     : "memory");
+      __syncwarp();
       wait_bounded(bar(B_DRAIN), 0, abort_flag, A.err, false);
     }
   } else {
     // ---------------------------------------------------------------- epilogue
-    const int q = warp & 3;  // TMEM lane quarter this warp may access
-    const int row = m_tile * BM + q * 32 + lane;
-    float best = -INFINITY;
-    int bi = -1;
+    const int q = warp & 3;            // TMEM lane quarter this warp may access
+    const int half = (warp - 2) >> 2;  // takes the 32-column chunks of this parity
+    uint32_t best[BN / 64];            // this lane's column of each chunk: running maximum (order key)
+    int bi[BN / 64];
+#pragma unroll
+    for (int j = 0; j < BN / 64; ++j) {
+      best[j] = kKeyNegInf;
+      bi[j] = -1;
+    }
+    bool ok = true;
     for (int t = 0; t < ntl; ++t) {
       const int a = t & 1;
-      const bool ok = wait_bounded(bar(B_ACCFULL + a), (t >> 1) & 1, abort_flag, A.err, true);
-      if (!__all_sync(0xffffffffu, ok)) break;
+      ok = wait_bounded(bar(B_ACCFULL + a), (t >> 1) & 1, abort_flag, A.err, true);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
       tc_fence_after();
-      const int v0 = (h_lo + 2 * t) * 128;
-      const int nc = wide(t) ? BN / 32 : BN / 64;
-#pragma unroll 1
-      for (int c = 0; c < nc; ++c) {
-        uint32_t r[32];
-        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + a * BN + c * 32, r);
-        tmem_wait_ld();
-        const int vc = v0 + c * 32;
-        if (vc + 32 <= A.V) {
+      const int v0 = (2 * (t_lo + t) + rank) * BV + q * 32;  // id of the warp's first lane
+      const bool in = v0 + lane < A.V;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float x = __uint_as_float(r[j]);
-            if (x > best) {
-              best = x;
-              bi = vc + j;
+      for (int j = 0; j < BN / 64; ++j) {
+        const int c = 2 * j + half;
+        if (c * 32 < A.nt) {
+          uint32_t r[32];
+          tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + a * BN + c * 32, r);
+          tmem_wait_ld();
+          uint32_t mk = 0u;
+          int ml = 0;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const uint32_t key = in ? order_key(__uint_as_float(r[i])) : 0u;
+            const uint32_t m = __reduce_max_sync(0xffffffffu, key);
+            const uint32_t who = __ballot_sync(0xffffffffu, key == m);
+            if (lane == i) {
+              mk = m;
+              ml = __ffs(who) - 1;
             }
           }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float x = __uint_as_float(r[j]);
-            if (vc + j < A.V && x > best) {
-              best = x;
-              bi = vc + j;
-            }
+          if (mk > best[j]) {
+            best[j] = mk;
+            bi[j] = v0 + ml;
           }
         }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_ACCEMPTY + a));
+      if (lane == 0) arrive_cluster(in_first_cta(bar(B_ACCEMPTY + a)));
     }
-    if (row < A.M && !*abort_flag) {
-      A.part_val[(int64_t)g * A.M + row] = best;
-      A.part_idx[(int64_t)g * A.M + row] = bi;
+    // the pair's maxima meet in the first CTA's ring, which nothing writes or
+    // reads any more once the last accumulator is complete: [8 quarters][256]
+    // keys, then ids
+    if (ok) {
+      const uint32_t base = in_first_cta(sb + kOffRing) + (rank * 4 + q) * BN * 4;
+#pragma unroll
+      for (int j = 0; j < BN / 64; ++j) {
+        const int c = 2 * j + half;
+        if (c * 32 < A.nt) {
+          st_cluster(base + (c * 32 + lane) * 4, best[j]);
+          st_cluster(base + 8 * BN * 4 + (c * 32 + lane) * 4, (uint32_t)bi[j]);
+        }
+      }
     }
   }
 
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
+  if (rank == 0 && !*abort_flag && (int)threadIdx.x < A.nt && n0 + (int)threadIdx.x < A.M) {
+    const uint32_t* keys = reinterpret_cast<const uint32_t*>(smem + kOffRing) + threadIdx.x;
+    const int* ids = reinterpret_cast<const int*>(keys) + 8 * BN;
+    uint32_t bk = 0u;
+    int b = -1;
+    for (int p = 0; p < 8; ++p) {
+      const uint32_t k = keys[p * BN];
+      const int i = ids[p * BN];
+      if (i >= 0 && (b < 0 || k > bk || (k == bk && i < b))) {
+        bk = k;
+        b = i;
+      }
+    }
+    A.part_key[(int64_t)g * A.M + n0 + threadIdx.x] = bk;
+    A.part_idx[(int64_t)g * A.M + n0 + threadIdx.x] = b;
+  }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
 
-// The first maximum over the vocab ranges, in vocab order.
+// The first maximum over the vocab ranges, a warp per row.
 __global__ void __launch_bounds__(256)
-lm_head_reduce_kernel(const float* __restrict__ part_val, const int32_t* __restrict__ part_idx, int groups, int M,
+lm_head_reduce_kernel(const uint32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx, int groups, int M,
                       int32_t* __restrict__ out, const int32_t* __restrict__ out_index) {
   pdl_begin();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (r >= M) return;
-  float best = -INFINITY;
-  int bi = -1;
-  for (int g = 0; g < groups; ++g) {
-    const float v = part_val[(int64_t)g * M + r];
+  uint32_t bk = 0u;  // a range without an id leaves 0, below every value's key
+  int b = INT_MAX;
+  for (int g = lane; g < groups; g += 32) {
     const int i = part_idx[(int64_t)g * M + r];
-    if (i >= 0 && (bi < 0 || v > best)) {
-      best = v;
-      bi = i;
+    const uint32_t k = i >= 0 ? part_key[(int64_t)g * M + r] : 0u;
+    if (k > bk) {  // ranges come in id order
+      bk = k;
+      b = i;
     }
   }
-  out[out_index ? out_index[r] : r] = bi < 0 ? 0 : bi;
+  const uint32_t m = __reduce_max_sync(0xffffffffu, bk);
+  const int id = __reduce_min_sync(0xffffffffu, bk == m ? b : INT_MAX);
+  if (lane == 0) out[out_index ? out_index[r] : r] = id == INT_MAX ? 0 : id;
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -297,16 +439,34 @@ bool make_rows_map(CUtensorMap* m, const void* base, uint64_t rows, int d, int b
 
 }  // namespace
 
+// Tiles of up to 256 hidden rows, a multiple of 32; the pairs left over by the
+// tiles split the vocabulary.  Of the tile counts at and just above the fewest,
+// the one with the least work on the busiest pair is taken, counted as its
+// vocab tiles x (columns + 100): measured at 817 rows, a vocab tile of 64 K
+// slices takes 19.7 / 17.6 / 15.0 / 14.0 / 13.2 us with 224 / 192 / 160 / 128 /
+// 96 columns, since below about 150 columns a slice costs what its barriers
+// and issue cost.  (1400 x 151936: 6 tiles of 256 1111 us, 10 of 160 1172; 257 x
+// 100001 x 2048: 2 of 160 90 us, 3 of 96 139.)
 LmPlan plan_lm_head(int rows, int vocab) {
   LmPlan p;
-  p.m_tiles = (rows + BM - 1) / BM;
-  p.h_tiles = (vocab + 127) / 128;
-  const int sms = num_sms();
-  int groups = sms / (p.m_tiles > 0 ? p.m_tiles : 1);
-  if (groups < 1) groups = 1;
-  if (groups > p.h_tiles) groups = p.h_tiles;
-  p.groups = groups;
-  p.ws_bytes = ((size_t)groups * rows * (sizeof(float) + sizeof(int32_t)) + 255) / 256 * 256;
+  p.v_tiles = (vocab + 2 * BV - 1) / (2 * BV);
+  const int pairs = std::max(1, num_sms() / 2);
+  const int fewest = std::max(1, (rows + BN - 1) / BN);
+  double least = 0;
+  for (int n = fewest; n < fewest + 8; ++n) {
+    const int nt = ((rows + n - 1) / n + 31) / 32 * 32;
+    const int tiles = std::max(1, (rows + nt - 1) / nt);
+    const int groups = std::min(std::max(1, pairs / tiles), p.v_tiles);
+    const int waves = (tiles * groups + pairs - 1) / pairs;
+    const double cost = (double)waves * ((p.v_tiles + groups - 1) / groups) * (std::max(nt, 128) + 100);
+    if (n == fewest || cost < least) {
+      least = cost;
+      p.nt = std::max(32, nt);
+      p.n_tiles = tiles;
+      p.groups = groups;
+    }
+  }
+  p.ws_bytes = ((size_t)p.groups * rows * (sizeof(uint32_t) + sizeof(int32_t)) + 255) / 256 * 256;
   return p;
 }
 
@@ -320,26 +480,29 @@ cudaError_t launch_lm_head_argmax(const LmPlan& p, const uint16_t* hidden, const
   if (e != cudaSuccess) return e;
   const uint64_t bit = 1ull << (dev & 63);
   if (!(attr_done.load() & bit)) {
-    e = cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax + 1024);
     if (e != cudaSuccess) return e;
     attr_done.fetch_or(bit);
   }
   CUtensorMap mh, mw;
-  if (!make_rows_map(&mh, hidden, (uint64_t)rows, d, BM) || !make_rows_map(&mw, w_lm, (uint64_t)vocab, d, BN))
+  if (!make_rows_map(&mh, hidden, (uint64_t)rows, d, p.nt / 2) || !make_rows_map(&mw, w_lm, (uint64_t)vocab, d, BV))
     return cudaErrorInvalidValue;
   LmArgs a;
   a.M = rows;
   a.d = d;
   a.V = vocab;
-  a.m_tiles = p.m_tiles;
+  a.nt = p.nt;
+  a.n_tiles = p.n_tiles;
   a.groups = p.groups;
-  a.h_tiles = p.h_tiles;
-  a.part_val = static_cast<float*>(workspace);
-  a.part_idx = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)p.groups * rows * sizeof(float));
+  a.v_tiles = p.v_tiles;
+  a.stages = stages_of(p.nt);
+  a.part_key = static_cast<uint32_t*>(workspace);
+  a.part_idx = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)p.groups * rows * sizeof(uint32_t));
   a.err = err;
-  e = launch_pdl(lm_head_argmax_kernel, dim3(p.m_tiles * p.groups), dim3(kThreads), kSmemBytes, s, mh, mw, a);
+  e = launch_pdl(lm_head_argmax_kernel, dim3(2 * p.n_tiles * p.groups), dim3(kThreads),
+                 1024 + kOffRing + a.stages * stage_bytes(p.nt), s, mh, mw, a);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(lm_head_reduce_kernel, dim3((rows + 255) / 256), dim3(256), 0, s, a.part_val, a.part_idx, p.groups,
+  e = launch_pdl(lm_head_reduce_kernel, dim3((rows + 7) / 8), dim3(256), 0, s, a.part_key, a.part_idx, p.groups,
                  rows, out, out_index);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

@@ -84,6 +84,25 @@ def test_lm_head_argmax_small_shapes(cure, rows, d, V):
     assert exact >= 0.8 * rows
 
 
+@pytest.mark.parametrize("rows,d,V", [(31, 64, 255), (32, 64, 257), (33, 128, 513), (255, 64, 5000), (256, 192, 5000),
+                                      (257, 64, 40000), (513, 128, 20000), (1281, 64, 2049), (2, 1024, 1)])
+def test_lm_head_argmax_tile_edges(cure, rows, d, V):
+    """Row counts around the tiles' multiples of 32 and 256 and vocabularies
+    around the pairs' 256-id tiles, one id included; fewer K slices than ring
+    stages and more."""
+    rng = np.random.default_rng(rows + V)
+    h = W.to_bf16(rng.standard_normal((rows, d)).astype(np.float32))
+    w = W.to_bf16((rng.standard_normal((V, d)) / np.sqrt(d)).astype(np.float32))
+    got = cure.cure_lm_head_argmax(h.to(DEV), w.to(DEV)).cpu().numpy()
+    assert cure.cure_device_error() == 0
+    if V == 1:
+        assert (got == 0).all()
+        return
+    sel = np.unique(np.concatenate([np.arange(min(rows, 40)), [rows - 1], rng.choice(rows, min(rows, 60), replace=False)]))
+    exact = _check(got[sel], W.bf16_to_f64(h)[sel], W.bf16_to_f64(w), d)
+    assert exact >= 0.8 * len(sel)
+
+
 def test_lm_head_argmax_more_m_tiles_than_sms(cure):
     """More 128-row tiles than SMs: one vocab range per tile and a grid of
     more than one wave."""
