@@ -108,24 +108,25 @@ constexpr uint32_t kColO = 256;  // O[m]:      columns 256 + m*128
 // within a 64-element half); kd and kd2 describe the two d halves of K.
 __device__ __forceinline__ void mma_s_group(uint32_t d, uint64_t qd, uint64_t kd, uint64_t kd2, uint32_t idesc) {
   asm volatile(
-      "{\n\t.reg .pred pf, pt;\n\t.reg .b64 a, b;\n\t"
+      "{\n\t.reg .pred pf, pt, el;\n\t.reg .b64 a, b;\n\t"
+      "elect.sync _|el, 0xffffffff;\n\t"
       "setp.ne.b32 pf, %4, %4;\n\t"
       "setp.eq.b32 pt, %4, %4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, pf;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, pf;\n\t"
       "add.s64 a, %1, 2;\n\tadd.s64 b, %2, 2;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, 4;\n\tadd.s64 b, %2, 4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, 6;\n\tadd.s64 b, %2, 6;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, %5;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, %6, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, %6, %3, pt;\n\t"
       "add.s64 a, %1, %5 + 2;\n\tadd.s64 b, %6, 2;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, %5 + 4;\n\tadd.s64 b, %6, 4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t"
       "add.s64 a, %1, %5 + 6;\n\tadd.s64 b, %6, 6;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t}\n" ::"r"(d),
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, pt;\n\t}\n" ::"r"(d),
       "l"(qd), "l"(kd), "r"(idesc), "r"(0), "n"(kQHalf >> 4), "l"(kd2)
       : "memory");
 }
@@ -134,17 +135,33 @@ __device__ __forceinline__ void mma_s_group(uint32_t d, uint64_t qd, uint64_t kd
 __device__ __forceinline__ void mma_pv_group(uint32_t d, uint32_t pa, uint64_t vd, uint32_t idesc,
                                              uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p0, pt;\n\t.reg .b64 b;\n\t.reg .b32 t;\n\t"
+      "{\n\t.reg .pred p0, pt, el;\n\t.reg .b64 b;\n\t.reg .b32 t;\n\t"
+      "elect.sync _|el, 0xffffffff;\n\t"
       "setp.ne.b32 p0, %4, 0;\n\t"
       "setp.eq.b32 pt, %4, %4;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p0;\n\t"
       "add.u32 t, %1, 8;\n\tadd.s64 b, %2, %5;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, pt;\n\t"
       "add.u32 t, %1, 16;\n\tadd.s64 b, %2, 2 * %5;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, pt;\n\t"
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, pt;\n\t"
       "add.u32 t, %1, 24;\n\tadd.s64 b, %2, 3 * %5;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, pt;\n\t}\n" ::"r"(d),
+      "@el tcgen05.mma.cta_group::1.kind::f16 [%0], [t], b, %3, pt;\n\t}\n" ::"r"(d),
       "r"(pa), "l"(vd), "r"(idesc), "r"(accumulate), "n"(kVChunk >> 4)
+      : "memory");
+}
+
+// Arrive on `bar` once the products this warp's elected lane issued are done.
+// The issuing warps run converged and elect the lane inside the asm: the
+// descriptors then stay in uniform registers, where a lane-0 branch moves each
+// operand of each product there (in the LM head's issuer, which steps the same
+// way, four products took 265 cycles to issue, now 124).  Graph-replayed:
+// 28 q / 4 kv heads, 16 sequences of 5001-8191 keys, trees of up to 65 nodes
+// 112 -> 107 us; 32 of 1024-8192 78.9 -> 77.4 us; 64 x 8 kv heads x 32768 keys
+// 1860 -> 1815 us.
+__device__ __forceinline__ void commit_elect(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred el;\n\telect.sync _|el, 0xffffffff;\n\t"
+      "@el tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar)
       : "memory");
 }
 
@@ -681,21 +698,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         if (sc > 0 && !wait_warp(bar(B_SFREE + m), (sc - 1) & 1u, abort_flag, A.err)) { ok = false; break; }
         if (!wait_warp(bar(B_KFULL + gt % NS), (gt / NS) & 1u, abort_flag, A.err)) { ok = false; break; }
         tc_fence_after();
-        if (lane == 0) {
-          // a paged cache tile interleaves the d halves per 8-key group
-          const bool pgd = A.kv.layout == 1 && s.t0 + j < s.nct;
-          const uint32_t ka = sb + kOffK + (gt % NS) * kTile;
-          const uint32_t sbo = pgd ? kPgGroup : 1024u, kh = pgd ? kPgHalf : kKVHalf;
-          mma_s_group(tmem + kColS + m * 64, qd, sdesc_sw128(ka, 16, sbo), sdesc_sw128(ka + kh, 16, sbo), idS);
-          mma_commit(bar(B_SFULL + m));
-          if (j == n - 1) mma_commit(bar(B_QEMPTY));  // the piece's last use of Q
-        }
-        __syncwarp();
+        // a paged cache tile interleaves the d halves per 8-key group
+        const bool pgd = A.kv.layout == 1 && s.t0 + j < s.nct;
+        const uint32_t ka = sb + kOffK + (gt % NS) * kTile;
+        const uint32_t sbo = pgd ? kPgGroup : 1024u, kh = pgd ? kPgHalf : kKVHalf;
+        mma_s_group(tmem + kColS + m * 64, qd, sdesc_sw128(ka, 16, sbo), sdesc_sw128(ka + kh, 16, sbo), idS);
+        commit_elect(bar(B_SFULL + m));
+        if (j == n - 1) commit_elect(bar(B_QEMPTY));  // the piece's last use of Q
         ++sc;
       }
     }
-    if (lane == 0) mma_commit(bar(B_DRAIN + m));
     __syncwarp();
+    commit_elect(bar(B_DRAIN + m));
     wait_bounded(bar(B_DRAIN + m), 0, abort_flag, A.err, false);
   } else if (warp == 11) {
     // ================================================================ PV issuer
@@ -719,17 +733,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
           ++oc;
         }
         tc_fence_after();
-        if (lane == 0) {
-          // V as an MN-major operand: the d halves LBO apart, 8-key groups SBO
-          // apart; a K = 16 step is 4 KiB in both layouts
-          const bool pgd = A.kv.layout == 1 && s.t0 + j < s.nct;
-          mma_pv_group(tmem + kColO + m * 128, tmem + kColP + m * 64 + (pc & 1u) * 32,
-                       sdesc_sw128(sb + kOffV + (gt % NS) * kTile, pgd ? kPgHalf : kVHalf,
-                                   pgd ? kPgGroup : 1024u),
-                       idO, j > 0 ? 1u : 0u);
-          mma_commit(bar(B_PVDONE + 2 * m + (pc & 1u)));
-        }
-        __syncwarp();
+        // V as an MN-major operand: the d halves LBO apart, 8-key groups SBO
+        // apart; a K = 16 step is 4 KiB in both layouts
+        const bool pgd = A.kv.layout == 1 && s.t0 + j < s.nct;
+        mma_pv_group(tmem + kColO + m * 128, tmem + kColP + m * 64 + (pc & 1u) * 32,
+                     sdesc_sw128(sb + kOffV + (gt % NS) * kTile, pgd ? kPgHalf : kVHalf,
+                                 pgd ? kPgGroup : 1024u),
+                     idO, j > 0 ? 1u : 0u);
+        commit_elect(bar(B_PVDONE + 2 * m + (pc & 1u)));
         ++pc;
         return true;
       };
@@ -737,12 +748,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         const uint32_t gt = gk0 + (uint32_t)j;
         if (!wait_warp(bar(B_VFULL + gt % NS), (gt / NS) & 1u, abort_flag, A.err)) { ok = false; break; }
         if (!issue_pv(0, pc0, oc0, j, gt) || (two && !issue_pv(1, pc1, oc1, j, gt))) { ok = false; break; }
-        if (lane == 0) mma_commit(bar(B_KVEMPTY + gt % NS));  // the tile's K and V are consumed
-        __syncwarp();
+        commit_elect(bar(B_KVEMPTY + gt % NS));  // the tile's K and V are consumed
       }
     }
-    if (lane == 0) mma_commit(bar(B_DRAIN + 2));
     __syncwarp();
+    commit_elect(bar(B_DRAIN + 2));
     wait_bounded(bar(B_DRAIN + 2), 0, abort_flag, A.err, false);
   } else {
     // ================================================================ softmax
