@@ -1117,7 +1117,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
 
   if constexpr (CLUSTER) {
     // ---------------------------------------------------------------- merge
-    // every CTA of the cluster takes 32 / csize float4 columns of all rows:
+    // the CTAs of the cluster take pairs of the 32 float4 columns in turn, all rows:
     // O = sum_p w_p O_p with w_p = 2^(lse_p - M) / sum_q 2^(lse_q - M)
     __syncwarp();
     cluster_sync();
@@ -1140,8 +1140,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
           wsum += w[p];
         }
         const float winv = 1.f / wsum;
-        const int ncol = 32 / sch.csize;  // 2, 4, 8 or 16
-        for (int c0 = sch.rank * ncol; c0 < (sch.rank + 1) * ncol; c0 += 2) {
+        for (int c0 = 2 * sch.rank; c0 < 32; c0 += 2 * sch.csize) {
           float acc[8] = {};
           const uint32_t col = sb + kOffK + (c0 * 2 * BM + tid) * 16;
 #pragma unroll
@@ -1313,16 +1312,17 @@ int max_clusters(int size) {
 //   stream-K: 16 + 1.5 per piece of a unit (its last piece merges the others'
 //             partials alone, through the workspace) + the CTA's tiles; the
 //             lengths of several sequences average about 3/4 of the longest;
-//   clusters: 11 + a CTA's share of the longest unit's tiles, if all units'
-//             clusters are resident at once; the merge runs on all CTAs of the
-//             unit through distributed shared memory.
+//   clusters: 10 + 0.1 per CTA + a CTA's share of the longest unit's tiles, if
+//             all units' clusters are resident at once; the merge runs on all
+//             CTAs of the unit through distributed shared memory.
 // The tiles are counted from the cache's capacity (the lengths are on the
-// device).  Measured, us per call, stream-K -> the cluster size chosen:
+// device).  Any size up to 16 is taken, whatever a GPC holds: 8 units fit in
+// clusters of 12, 16 in 7, 32 in 4.  Measured, us per call, stream-K -> clusters:
 //   1 sequence x 8 kv heads of 4 query heads, 300 / 4096 / 16384 keys
-//                                                  17.0 / 26.5 / 50.8 -> 9.7 / 15.4 / 34.5 (8)
-//   1 x 8, 65536 keys                              75.9 stays (8: 108)
-//   1 x 4 of 7, 4096 keys, in place                34.4 -> 17.7 (16)
-//   4 x 8 of 4, 1000-4096 keys                     30.0 -> 21.3 (4)
+//                                                  17.0 / 26.5 / 50.8 -> 9.7 / 14.1 / 26.7
+//   1 x 16 of 1, 4096 keys                         29.6 -> 16.6 (powers of two only: 20.2)
+//   1 x 4 of 7, 4096 keys, in place                34.4 -> 17.6
+//   4 x 8 of 4, 1000-4096 keys                     30.0 -> 21.0
 //   8 x 8 of 8, 1024-4096 keys, two M tiles        38.2 stays (2: 40.9)
 //   16 x 4 of 7, 1024-8192 keys                    50.5 stays (2: 66.9)
 int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
@@ -1332,8 +1332,8 @@ int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
   const float ctas = std::min<float>((float)sms, (float)units * (tiles + kAttnUnitCost) / kAttnMinTiles);
   float best = 16.f + 1.5f * ctas / units + tile * (ragged ? 0.75f : 1.f) * tiles * units / ctas;
   int size = 0;
-  for (int c = 2; c <= kAttnMaxCluster; c *= 2) {
-    const float t = 11.f + tile * tiles / c;
+  for (int c = 2; c <= kAttnMaxCluster; ++c) {
+    const float t = 10.f + 0.1f * c + tile * tiles / c;
     if (t < best && units <= max_clusters(c)) {
       best = t;
       size = c;
