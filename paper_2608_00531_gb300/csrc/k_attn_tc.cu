@@ -58,6 +58,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "attn_common.cuh"
 #include "tc_ptx.cuh"
@@ -282,15 +283,18 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float ld_cluster_f32(uint32_t a) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+__device__ __forceinline__ float ld_cluster_f32(uint32_t a, bool on, float off) {
+  float v = off;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.shared::cluster.f32 %0, [%1];\n\t}\n"
+               : "+f"(v) : "r"(a), "r"((int)on));
   return v;
 }
-__device__ __forceinline__ float4 ld_cluster_v4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t a, bool on) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+      "@p ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}\n"
+      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w) : "r"(a), "r"((int)on));
   return v;
 }
 
@@ -385,8 +389,8 @@ struct Sched {
     s.rg = uib / Hkv;
     s.h = uib % Hkv;
     s.u = unit;
-    s.t0 = (int)((long long)rank * s.T / csize);
-    s.t1 = (int)((long long)(rank + 1) * s.T / csize);
+    s.t0 = (int)((unsigned)rank * (unsigned)s.T / (unsigned)csize);  // T < 2^25
+    s.t1 = (int)((unsigned)(rank + 1) * (unsigned)s.T / (unsigned)csize);
     s.parts = csize;
     s.part = rank;
     s.slot = 0;
@@ -572,15 +576,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       auto load_q = [&]() -> bool {
         if (!wait_warp(bar(B_QEMPTY), (qc & 1u) ^ 1u, abort_flag, A.err)) return false;
         ++qc;
-        if (lane == 0) {
-          mbar_arrive_expect_tx(bar(B_QFULL), 4 * qbytes);
-          for (int m = 0; m < 2; ++m) {
-            const int node0 = (2 * s.rg + m) * npb;
-            for (int hf = 0; hf < 2; ++hf)
-              tma_load_4d(sb + kOffQ + (2 * m + hf) * kQHalf, &tm_q, bar(B_QFULL), hf * 64, 0, s.h,
-                          s.b * A.n_max + node0);
-          }
-        }
+        if (lane == 0) mbar_arrive_expect_tx(bar(B_QFULL), 4 * qbytes);
+        __syncwarp();
+        if (lane < 4)  // M tile lane / 2, d half lane % 2
+          tma_load_4d(sb + kOffQ + lane * kQHalf, &tm_q, bar(B_QFULL), (lane & 1) * 64, 0, s.h,
+                      s.b * A.n_max + (2 * s.rg + (lane >> 1)) * npb);
         __syncwarp();
         return true;
       };
@@ -654,13 +654,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         issue_k(sb + kOffK + st * kTile, bar(B_KFULL + st));
         __syncwarp();
         ++k_issued;
+        // (a cluster's CTA has one piece: its Q goes between the first K and V)
+        if (CLUSTER && t == s.t0 && !load_q()) { ok = false; break; }
         if (lane == 0) mbar_arrive_expect_tx(bar(B_VFULL + st), kTile);
         __syncwarp();
         issue_v(sb + kOffV + st * kTile, bar(B_VFULL + st));
         __syncwarp();
         ++v_issued;
         ++gk;
-        if (t == s.t0 && !load_q()) { ok = false; break; }
+        if (!CLUSTER && t == s.t0 && !load_q()) { ok = false; break; }
       }
     }
     if (*abort_flag) {  // let copies in flight land before the CTA's smem goes away
@@ -1117,50 +1119,66 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
 
   if constexpr (CLUSTER) {
     // ---------------------------------------------------------------- merge
-    // the CTAs of the cluster take pairs of the 32 float4 columns in turn, all rows:
-    // O = sum_p w_p O_p with w_p = 2^(lse_p - M) / sum_q 2^(lse_q - M)
+    // the CTAs of the cluster take the 32 float4 columns in turn, and within a CTA
+    // its three groups of 128 threads; a thread merges one row of a column:
+    // O = sum_p w_p O_p with w_p = 2^(lse_p - M) / sum_q 2^(lse_q - M), all
+    // CTAs' loads in flight together (predicated, not branched around; a CTA
+    // of weight 0 may have written no O and is not read)
     __syncwarp();
     cluster_sync();
-    if (takes_part && warp < 8) {
+    // up to 16 loads a thread in flight: P CTAs (at least csize) x 16 / P columns
+    auto merge = [&](auto ptag) {
+      constexpr int P = decltype(ptag)::value, C = kAttnMaxCluster / P;
       const Seg s = sch.at(0, 1);
-      const int row = tid & 127, m = warp >> 2;
+      // one M tile: three groups of 128 threads share its columns; two: a group each
+      const bool two = active1(s);
+      const int row = tid & 127, grp = two ? 0 : tid >> 7, ngrp = two ? 1 : 3, m = two ? tid >> 7 : 0;
       const int node = (2 * s.rg + m) * npb + row / G, gh = row % G;
-      if (row < npb * G && node < s.n) {
-        const uint32_t lse_a = sb + kOffK + 32 * 2 * BM * 16 + tid * 4;
-        float w[kAttnMaxCluster];  // log-sum-exps, then weights (0: no tile of the unit, no O written)
-        float M = -INFINITY, wsum = 0.f;
+      if (m > 1 || row >= npb * G || node >= s.n) return;
+      const uint32_t lse_a = sb + kOffK + 32 * 2 * BM * 16 + (m * BM + row) * 4;
+      float w[P];  // log-sum-exps, then weights
+      float M = -INFINITY, wsum = 0.f;
 #pragma unroll
-        for (int p = 0; p < kAttnMaxCluster; ++p)
-          w[p] = p < sch.csize ? ld_cluster_f32(map_rank(lse_a, p)) : -INFINITY;
+      for (int p = 0; p < P; ++p) w[p] = ld_cluster_f32(map_rank(lse_a, p), p < sch.csize, -INFINITY);
 #pragma unroll
-        for (int p = 0; p < kAttnMaxCluster; ++p) M = fmaxf(M, w[p]);
+      for (int p = 0; p < P; ++p) M = fmaxf(M, w[p]);
 #pragma unroll
-        for (int p = 0; p < kAttnMaxCluster; ++p) {
-          w[p] = w[p] == -INFINITY ? 0.f : ex2(w[p] - M);
-          wsum += w[p];
+      for (int p = 0; p < P; ++p) {
+        w[p] = w[p] == -INFINITY ? 0.f : ex2(w[p] - M);
+        wsum += w[p];
+      }
+      const float winv = 1.f / wsum;
+      uint16_t* orow = A.out + (((int64_t)s.b * A.n_max + node) * A.heads_q + s.h * G + gh) * D;
+      const int step = sch.csize * ngrp;
+      for (int c = sch.rank + sch.csize * grp; c < 32; c += C * step) {
+        float4 o[C][P];
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+          const uint32_t col = sb + kOffK + ((c + j * step) * 2 * BM + m * BM + row) * 16;
+#pragma unroll
+          for (int p = 0; p < P; ++p) o[j][p] = ld_cluster_v4(map_rank(col, p), w[p] > 0.f && c + j * step < 32);
         }
-        const float winv = 1.f / wsum;
-        for (int c0 = 2 * sch.rank; c0 < 32; c0 += 2 * sch.csize) {
-          float acc[8] = {};
-          const uint32_t col = sb + kOffK + (c0 * 2 * BM + tid) * 16;
 #pragma unroll
-          for (int p = 0; p < kAttnMaxCluster; ++p) {
-            if (w[p] > 0.f) {
-              const float4 a = ld_cluster_v4(map_rank(col, p)), b = ld_cluster_v4(map_rank(col, p) + 2 * BM * 16);
-              const float wp = w[p] * winv;
-              acc[0] += wp * a.x; acc[1] += wp * a.y; acc[2] += wp * a.z; acc[3] += wp * a.w;
-              acc[4] += wp * b.x; acc[5] += wp * b.y; acc[6] += wp * b.z; acc[7] += wp * b.w;
-            }
+        for (int j = 0; j < C; ++j) {
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int p = 0; p < P; ++p) {
+            const float wp = w[p] * winv;
+            acc.x += wp * o[j][p].x;
+            acc.y += wp * o[j][p].y;
+            acc.z += wp * o[j][p].z;
+            acc.w += wp * o[j][p].w;
           }
-          uint4 v;
-          v.x = pack_bf16(acc[0], acc[1]);
-          v.y = pack_bf16(acc[2], acc[3]);
-          v.z = pack_bf16(acc[4], acc[5]);
-          v.w = pack_bf16(acc[6], acc[7]);
-          *reinterpret_cast<uint4*>(A.out + (((int64_t)s.b * A.n_max + node) * A.heads_q + s.h * G + gh) * D +
-                                    c0 * 4) = v;
+          if (c + j * step < 32)
+            *reinterpret_cast<uint2*>(orow + (c + j * step) * 4) =
+                make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
         }
       }
+    };
+    if (takes_part) {
+      if (sch.csize <= 4) merge(std::integral_constant<int, 4>());
+      else if (sch.csize <= 8) merge(std::integral_constant<int, 8>());
+      else merge(std::integral_constant<int, 16>());
     }
     __syncwarp();
     cluster_sync();  // the peers have read this CTA's shared memory
@@ -1312,19 +1330,23 @@ int max_clusters(int size) {
 //   stream-K: 16 + 1.5 per piece of a unit (its last piece merges the others'
 //             partials alone, through the workspace) + the CTA's tiles; the
 //             lengths of several sequences average about 3/4 of the longest;
-//   clusters: 10 + 0.1 per CTA + a CTA's share of the longest unit's tiles, if
+//   clusters: 9 + 0.1 per CTA + a CTA's share of the longest unit's tiles, if
 //             all units' clusters are resident at once; the merge runs on all
 //             CTAs of the unit through distributed shared memory.
 // The tiles are counted from the cache's capacity (the lengths are on the
 // device).  Any size up to 16 is taken, whatever a GPC holds: 8 units fit in
 // clusters of 12, 16 in 7, 32 in 4.  Measured, us per call, stream-K -> clusters:
 //   1 sequence x 8 kv heads of 4 query heads, 300 / 4096 / 16384 keys
-//                                                  17.0 / 26.5 / 50.8 -> 9.7 / 14.1 / 26.7
-//   1 x 16 of 1, 4096 keys                         29.6 -> 16.6 (powers of two only: 20.2)
-//   1 x 4 of 7, 4096 keys, in place                34.4 -> 17.6
-//   4 x 8 of 4, 1000-4096 keys                     30.0 -> 21.0
+//                                                  17.0 / 26.5 / 50.8 -> 8.8 / 13.0 / 26.0
+//   1 x 16 of 1, 4096 keys                         29.6 -> 15.5
+//   1 x 4 of 7, 4096 keys, in place                34.4 -> 16.3
+//   4 x 8 of 4, 1000-4096 keys                     30.0 -> 19.9
 //   8 x 8 of 8, 1024-4096 keys, two M tiles        38.2 stays (2: 40.9)
 //   16 x 4 of 7, 1024-8192 keys                    50.5 stays (2: 66.9)
+// What a cluster call spends at 4096 keys, from one CTA's clock stamps (us):
+// schedule 0.6, first K and Q 1.9, 5.5 tiles 3.5, the last product 0.4, its
+// results into shared memory 0.5, waiting for the peers 1.7, the merge (3.2 with
+// loads branched around or in small batches, about 2 now), leaving 0.9.
 int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
   if (units < 1 || set_attributes() != cudaSuccess) return 0;
   const int sms = num_sms();
@@ -1333,7 +1355,7 @@ int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
   float best = 16.f + 1.5f * ctas / units + tile * (ragged ? 0.75f : 1.f) * tiles * units / ctas;
   int size = 0;
   for (int c = 2; c <= kAttnMaxCluster; ++c) {
-    const float t = 10.f + 0.1f * c + tile * tiles / c;
+    const float t = 9.f + 0.1f * c + tile * tiles / c;
     if (t < best && units <= max_clusters(c)) {
       best = t;
       size = c;
