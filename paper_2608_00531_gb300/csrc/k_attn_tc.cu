@@ -91,7 +91,7 @@ constexpr int kOffMisc = kOffV + NS * kTile;      // 196608
 enum {
   B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_VFULL = B_KFULL + NS, B_KVEMPTY = B_VFULL + NS,
   B_SFULL = B_KVEMPTY + NS, B_SFREE = B_SFULL + 2, B_PFULL = B_SFREE + 2, B_PVDONE = B_PFULL + 4,
-  B_OFREE = B_PVDONE + 4, B_DRAIN = B_OFREE + 2, kNumBars = B_DRAIN + 3
+  B_OFREE = B_PVDONE + 4, B_DRAIN = B_OFREE + 2, B_Q1FULL = B_DRAIN + 3, B_Q1EMPTY, kNumBars
 };
 constexpr int kOffTmemSlot = kOffMisc + 8 * kNumBars;
 constexpr int kOffAbort = kOffTmemSlot + 4;
@@ -400,6 +400,8 @@ struct Sched {
   int unit, rank, csize;  // CLUSTER: this cluster's unit, this CTA's rank, the cluster size
 };
 
+enum { kStreamK = 0, kCluster = 1, kPingPong = 2 };
+
 // INPLACE: the in-place layout (no tree tensors; node j's rows at cache slot
 // L + j), a template parameter so that the separate-tensor kernel carries
 // none of its tests.
@@ -407,11 +409,17 @@ struct Sched {
 // CLUSTER: one unit per cluster of CTAs, merged through distributed shared
 // memory, for problems with too few units to fill the GPU (see
 // attn_cluster_size for when).
-template <bool INPLACE, bool CLUSTER>
+//
+// PINGPONG: stream-K where every unit fits one M tile (n_max <= npb).  The two
+// M tile slots (Q, S, P, O and a softmax warpgroup each) then take a CTA's
+// pieces in turn, so that a piece's first products and softmax run under the
+// previous piece's epilogue, and its Q is loaded while that one still uses its own.
+template <bool INPLACE, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                     const __grid_constant__ CUtensorMap tm_tk, const __grid_constant__ CUtensorMap tm_tv,
                     const __grid_constant__ CUtensorMap tm_q, const AttnArgs A) {
+  constexpr bool CLUSTER = MODE == kCluster, PINGPONG = MODE == kPingPong;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t sb = smem_u32(smem);
@@ -423,14 +431,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   const int npb = BM / G;  // tree nodes per M tile
   const Bar bar{sb + kOffMisc};
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffAbort);
-  volatile int* last_flag = reinterpret_cast<volatile int*>(smem + kOffLast);
   int* tiles_start = reinterpret_cast<int*>(smem + kOffPrefix);
   int* units_start = tiles_start + (kAttnMaxBatch + 1);
 
   // ---------------------------------------------------------------- set-up
   if (tid == 0) {
     mbar_init(bar(B_QFULL), 1);
-    mbar_init(bar(B_QEMPTY), 2);
+    mbar_init(bar(B_QEMPTY), PINGPONG ? 1 : 2);
+    mbar_init(bar(B_Q1FULL), 1);
+    mbar_init(bar(B_Q1EMPTY), 1);
     for (int i = 0; i < NS; ++i) {
       mbar_init(bar(B_KFULL + i), 1);
       mbar_init(bar(B_VFULL + i), 1);
@@ -562,7 +571,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       if (s.t1 <= s.t0) continue;
       // the next piece's Q boxes are prefetched into L2 now, so that its Q
       // load at the piece boundary is served from L2
-      if (g < g_end && lane == 0) {
+      if (!PINGPONG && g < g_end && lane == 0) {
         const Seg nx = sch.at(g, g_end);
         if (nx.t1 > nx.t0) {
           for (int m = 0; m < (active1(nx) ? 2 : 1); ++m)
@@ -574,6 +583,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       // is requested after the piece's first K/V tile, whose ring stage frees
       // up independently, so that the ring refills across the piece boundary
       auto load_q = [&]() -> bool {
+        if constexpr (PINGPONG) {  // into the slot of the piece before the last
+          const uint32_t slot = qc & 1u, full = bar(slot ? B_Q1FULL : B_QFULL);
+          if (!wait_warp(bar(slot ? B_Q1EMPTY : B_QEMPTY), ((qc >> 1) & 1u) ^ 1u, abort_flag, A.err)) return false;
+          ++qc;
+          if (lane == 0) mbar_arrive_expect_tx(full, 2 * qbytes);
+          __syncwarp();
+          if (lane < 2)
+            tma_load_4d(sb + kOffQ + (2 * slot + lane) * kQHalf, &tm_q, full, lane * 64, 0, s.h,
+                        s.b * A.n_max + 2 * s.rg * npb);
+          __syncwarp();
+          return true;
+        }
         if (!wait_warp(bar(B_QEMPTY), (qc & 1u) ^ 1u, abort_flag, A.err)) return false;
         ++qc;
         if (lane == 0) mbar_arrive_expect_tx(bar(B_QFULL), 4 * qbytes);
@@ -654,15 +675,16 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         issue_k(sb + kOffK + st * kTile, bar(B_KFULL + st));
         __syncwarp();
         ++k_issued;
-        // (a cluster's CTA has one piece: its Q goes between the first K and V)
-        if (CLUSTER && t == s.t0 && !load_q()) { ok = false; break; }
+        // a cluster's CTA has one piece, and a ping-pong piece's Q slot is long
+        // free: Q goes between the first K and V
+        if (MODE != kStreamK && t == s.t0 && !load_q()) { ok = false; break; }
         if (lane == 0) mbar_arrive_expect_tx(bar(B_VFULL + st), kTile);
         __syncwarp();
         issue_v(sb + kOffV + st * kTile, bar(B_VFULL + st));
         __syncwarp();
         ++v_issued;
         ++gk;
-        if (!CLUSTER && t == s.t0 && !load_q()) { ok = false; break; }
+        if (MODE == kStreamK && t == s.t0 && !load_q()) { ok = false; break; }
       }
     }
     if (*abort_flag) {  // let copies in flight land before the CTA's smem goes away
@@ -670,7 +692,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         wait_bounded(bar(B_KFULL + i % NS), (i / NS) & 1u, abort_flag, A.err, false);
       for (uint32_t i = (v_issued > NS ? v_issued - NS : 0); i < v_issued; ++i)
         wait_bounded(bar(B_VFULL + i % NS), (i / NS) & 1u, abort_flag, A.err, false);
-      if (qc > 0) wait_bounded(bar(B_QFULL), (qc - 1) & 1u, abort_flag, A.err, false);
+      if constexpr (PINGPONG) {
+        if (qc > 0) wait_bounded(bar(B_QFULL), (((qc + 1) >> 1) - 1) & 1u, abort_flag, A.err, false);
+        if (qc > 1) wait_bounded(bar(B_Q1FULL), ((qc >> 1) - 1) & 1u, abort_flag, A.err, false);
+      } else if (qc > 0) {
+        wait_bounded(bar(B_QFULL), (qc - 1) & 1u, abort_flag, A.err, false);
+      }
     }
   } else if (warp == 9 || warp == 10) {
     // ================================================================ S issuers
@@ -687,9 +714,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       const int n = s.t1 - s.t0;
       const uint32_t gk0 = gk;
       gk += (uint32_t)n;
-      if (!wait_warp(bar(B_QFULL), qc & 1u, abort_flag, A.err)) { ok = false; break; }
-      ++qc;
-      if (!(m == 0 || active1(s))) {  // no rows in this M tile: Q is free at once
+      if constexpr (PINGPONG) {  // qc: pieces; those of this warp's slot
+        const uint32_t q = qc++;
+        if ((int)(q & 1u) != m) continue;
+        if (!wait_warp(bar(m ? B_Q1FULL : B_QFULL), (q >> 1) & 1u, abort_flag, A.err)) { ok = false; break; }
+      } else {
+        if (!wait_warp(bar(B_QFULL), qc & 1u, abort_flag, A.err)) { ok = false; break; }
+        ++qc;
+      }
+      if (!PINGPONG && !(m == 0 || active1(s))) {  // no rows in this M tile: Q is free at once
         if (lane == 0) mbar_arrive(bar(B_QEMPTY));
         __syncwarp();
         continue;
@@ -706,7 +739,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         const uint32_t sbo = pgd ? kPgGroup : 1024u, kh = pgd ? kPgHalf : kKVHalf;
         mma_s_group(tmem + kColS + m * 64, qd, sdesc_sw128(ka, 16, sbo), sdesc_sw128(ka + kh, 16, sbo), idS);
         commit_elect(bar(B_SFULL + m));
-        if (j == n - 1) commit_elect(bar(B_QEMPTY));  // the piece's last use of Q
+        if (j == n - 1) commit_elect(bar(PINGPONG && m ? B_Q1EMPTY : B_QEMPTY));  // the piece's last use of Q
         ++sc;
       }
     }
@@ -718,7 +751,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     // O_m += P_m V for both M tiles as soon as the softmax has published P_m;
     // the K/V stage is released after the tile's last PV product
     constexpr uint32_t idO = idesc_bf16_f32(BM, D, true);
-    uint32_t gk = 0, pc0 = 0, pc1 = 0, oc0 = 0, oc1 = 0;
+    uint32_t gk = 0, pc0 = 0, pc1 = 0, oc0 = 0, oc1 = 0, pieces = 0;
     bool ok = true;
     for (long long g = g_begin; ok && g < g_end;) {
       const Seg s = sch.at(g, g_end);
@@ -728,6 +761,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       const uint32_t gk0 = gk;
       gk += (uint32_t)n;
       const bool two = active1(s);
+      const bool slot1 = PINGPONG && (pieces++ & 1u);
       auto issue_pv = [&](int m, uint32_t& pc, uint32_t& oc, int j, uint32_t gt) -> bool {
         if (!wait_warp(bar(B_PFULL + 2 * m + (pc & 1u)), (pc >> 1) & 1u, abort_flag, A.err)) return false;
         if (j == 0) {  // O_m holds the previous piece until its epilogue has read it
@@ -749,7 +783,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       for (int j = 0; ok && j < n; ++j) {
         const uint32_t gt = gk0 + (uint32_t)j;
         if (!wait_warp(bar(B_VFULL + gt % NS), (gt / NS) & 1u, abort_flag, A.err)) { ok = false; break; }
-        if (!issue_pv(0, pc0, oc0, j, gt) || (two && !issue_pv(1, pc1, oc1, j, gt))) { ok = false; break; }
+        if constexpr (PINGPONG) {
+          if (!(slot1 ? issue_pv(1, pc1, oc1, j, gt) : issue_pv(0, pc0, oc0, j, gt))) { ok = false; break; }
+        } else {
+          if (!issue_pv(0, pc0, oc0, j, gt) || (two && !issue_pv(1, pc1, oc1, j, gt))) { ok = false; break; }
+        }
         commit_elect(bar(B_KVEMPTY + gt % NS));  // the tile's K and V are consumed
       }
     }
@@ -762,8 +800,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     const int row = tid & 127; // row within the M tile = TMEM lane
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float c = A.scale_log2;
-    uint32_t sc = 0, gk = 0;
+    uint32_t sc = 0, gk = 0, pieces = 0;
     bool ok = true;
+    // the warps that share a piece's epilogue, its thread 0 and its flag
+    auto sync_epilogue = [&]() {
+      if constexpr (PINGPONG) asm volatile("bar.sync %0, 128;" ::"r"(1 + m) : "memory");
+      else named_sync_softmax();
+    };
+    const bool first = PINGPONG ? row == 0 : tid == 0;
+    volatile int* last_flag = reinterpret_cast<volatile int*>(smem + kOffLast) + (PINGPONG ? m : 0);
     for (long long g = g_begin; g < g_end;) {
       const Seg s = sch.at(g, g_end);
       g = s.next;
@@ -771,8 +816,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       const int n = s.t1 - s.t0;
       const uint32_t gk0 = gk;
       gk += (uint32_t)n;
-      const bool act = m == 0 || active1(s);
-      const int node0 = (2 * s.rg + m) * npb;
+      if (PINGPONG && (int)(pieces++ & 1u) != m) continue;
+      const bool act = PINGPONG || m == 0 || active1(s);
+      const int node0 = (2 * s.rg + (PINGPONG ? 0 : m)) * npb;
       const int node = node0 + row / G, gh = row % G;
       const bool vrow = act && row < npb * G && node < s.n;
       float m_run = -INFINITY, l_run = 0.f;
@@ -970,7 +1016,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
       // a piece's partial: fp32 float4 columns [32][256 rows], so that the 32
       // rows of a warp touch 512 contiguous bytes at every column
-      const int prow = m * BM + row;
+      const int prow = PINGPONG ? row : m * BM + row;
       float4* pslot = reinterpret_cast<float4*>(A.ws_o) + (int64_t)(s.slot + s.part) * (32 * 2 * BM);
       uint16_t* orow =
           A.out + (((int64_t)s.b * A.n_max + min(node, A.n_max - 1)) * A.heads_q + s.h * G + gh) * D;
@@ -1003,10 +1049,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         // its partial, publishes (release fence + counter), and merges if the
         // counter says it came last.  O_m is released after the merge.
         const float lse_own = m_run + log2f(l_run);
-        named_sync_softmax();
-        if (tid == 0)
+        sync_epilogue();
+        if (first)
           *last_flag = (!*abort_flag && count_of(ld_acquire(A.cnt + s.u), A.tag) == s.parts - 1) ? 2 : 0;
-        named_sync_softmax();
+        sync_epilogue();
         int last = *last_flag;
         if (last != 2) {
           if (act && ok) {
@@ -1026,8 +1072,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
           }
           if (vrow && ok) A.ws_lse[(int64_t)(s.slot + s.part) * (2 * BM) + prow] = lse_own;
           __threadfence();
-          named_sync_softmax();
-          if (tid == 0) {
+          sync_epilogue();
+          if (first) {
             int l = 0;
             if (!*abort_flag) {
               l = arrive(A.cnt + s.u, A.tag) == s.parts;
@@ -1035,9 +1081,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
             }
             *last_flag = l;
           }
-          named_sync_softmax();
+          sync_epilogue();
           last = *last_flag;
-        } else if (tid == 0) {
+        } else if (first) {
           A.cnt[s.u] = 0;  // a completed unit leaves a zero word behind
         }
         if (last && act && ok) {
@@ -1269,8 +1315,9 @@ namespace {
 
 using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                         const AttnArgs);
-constexpr Kernel kKernels[4] = {tree_attn_tc_kernel<false, false>, tree_attn_tc_kernel<true, false>,
-                                tree_attn_tc_kernel<false, true>, tree_attn_tc_kernel<true, true>};
+constexpr Kernel kKernels[3][2] = {{tree_attn_tc_kernel<false, kStreamK>, tree_attn_tc_kernel<true, kStreamK>},
+                                   {tree_attn_tc_kernel<false, kCluster>, tree_attn_tc_kernel<true, kCluster>},
+                                   {tree_attn_tc_kernel<false, kPingPong>, tree_attn_tc_kernel<true, kPingPong>}};
 
 // Dynamic shared memory and clusters above the portable size, once per device.
 cudaError_t set_attributes() {
@@ -1280,10 +1327,12 @@ cudaError_t set_attributes() {
   if (e != cudaSuccess) return e;
   const uint64_t bit = 1ull << (dev & 63);
   if (done.load() & bit) return cudaSuccess;
-  for (Kernel k : kKernels) {
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
+  for (const auto& mode : kKernels) {
+    for (Kernel k : mode) {
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
   }
   done.fetch_or(bit);
   return cudaSuccess;
@@ -1313,7 +1362,7 @@ int max_clusters(int size) {
   if (n == 0) {
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config(attr, dim3(size), size);
-    if (cudaOccupancyMaxActiveClusters(&n, kKernels[2], &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, kKernels[kCluster][0], &cfg) != cudaSuccess) {
       cudaGetLastError();
       n = 0;
     }
@@ -1397,7 +1446,14 @@ cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see pdl_begin()
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, kKernels[(A.inplace ? 1 : 0) + (A.cluster > 0 ? 2 : 0)], mk, mv, mtk, mtv, mq, a);
+  // Ping-pong where every unit fits one M tile and a CTA has at least 1.5 units
+  // on average: it hides the pieces' starts and ends (64 sequences x 8 kv heads x
+  // 200-300 keys 46.6 -> 39.9 us, 16 x 16 x 500-900 36.4 -> 33.0, 32 x 8 x 1024-8192
+  // 111.8 -> 108.6), and with fewer, longer pieces its tiles cost 1 % more (16 x 8 x
+  // 1024-8192, 0.84 units a CTA, 61.5 -> 62.2; 20 x 8 x 3000-9000, 1.05, 84.9 -> 86.2).
+  const bool one_tile = A.n_max <= BM / A.G;
+  const int mode = A.cluster > 0 ? kCluster : one_tile && 2 * (int64_t)A.units_max >= 3 * (int64_t)grid.x ? kPingPong : kStreamK;
+  e = cudaLaunchKernelEx(&cfg, kKernels[mode][A.inplace ? 1 : 0], mk, mv, mtk, mtv, mq, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

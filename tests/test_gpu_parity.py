@@ -450,6 +450,38 @@ def test_tree_attn_workspace_contents_do_not_matter(cure):
                 assert np.abs(got[b, :n] - ref[b, :n]).max() <= 1e-2, (fill, b)
 
 
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("Hq,Hkv", [(32, 8), (8, 8), (40, 8)])
+def test_tree_attn_many_one_tile_units(cure, Hq, Hkv, paged, in_place):
+    """At least 1.5 units per SM that fit one M tile each: a CTA's pieces take
+    the two tile slots in turn, whole and split units, one-tile pieces (empty
+    caches) and longer ones mixed; called twice on one garbage workspace."""
+    B = 30
+    rng = np.random.default_rng(Hq)
+    lens = [0, 1, 63, 64, 65, 1500] + [int(v) for v in rng.integers(0, 500, B - 6)]
+    if in_place:
+        t, q, kc, vc, L, table, npages = _in_place_case(B, 12, 8, Hq, Hkv, lens, paged, seed=Hq)
+        tk = tv = None
+    else:
+        t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 12, 8, Hq, Hkv, lens, paged, 1.0, 1.0, seed=Hq)
+    assert q.shape[1] <= 128 // (Hq // Hkv)
+    kv = cure.kv_desc(Hkv, 128, table.shape[1], torch.from_numpy(table).to(DEV), 16, npages) if paged else \
+        cure.kv_desc(Hkv, 128, kc.shape[1])
+    ws = torch.randint(0, 256, (cure.cure_tree_attn_workspace_size(B, q.shape[1], Hq, kv),), dtype=torch.uint8,
+                       device=DEV, generator=torch.Generator(device=DEV).manual_seed(3))
+    dev = [x.to(DEV) if x is not None else None for x in (q, tk, tv, kc, vc)]
+    ref = oracle.tree_attn(_f64(q), None if tk is None else _f64(tk), None if tv is None else _f64(tv), _f64(kc),
+                           _f64(vc), L, t["n_nodes"], t["anc"], 1.0 / math.sqrt(128), table, 16)
+    for _ in range(2):
+        got = cure.cure_tree_attn(*dev, kv, torch.from_numpy(L).to(DEV),
+                                  torch.from_numpy(t["n_nodes"].astype(np.int32)).to(DEV),
+                                  torch.from_numpy(t["anc"].view(np.int64)).to(DEV), 1.0 / math.sqrt(128),
+                                  workspace=ws).float().cpu().numpy()
+        assert cure.cure_device_error() == 0
+        _cmp_attn(got, ref, t)
+
+
 @pytest.mark.parametrize("paged", [False, True])
 def test_tree_attn_split_units_on_garbage_workspace(cure, paged):
     """96 units, too many for a cluster each: the units cut by the stream-K
