@@ -19,7 +19,7 @@
 //            CTAs' TMEM; two accumulators alternate between vocab tiles;
 //   warps 2-9 epilogue (each CTA): a TMEM lane is a vocab id, a column a hidden
 //            row; the warp takes each column's maximum and its first lane (a
-//            redux and a ballot), and the lane that keeps the column replaces
+//            float redux and a ballot), and the lane that keeps the column replaces
 //            its running (max, id) when strictly greater, so the lowest id
 //            wins ties.
 // The pair merges its 8 lane quarters through the first CTA's shared memory and
@@ -29,15 +29,18 @@
 // leaves.
 //
 // What bounds it: with one tile of rows the weight's bytes (21 x 4096 x 128256:
-// 160 us, 6.6 TB/s); with several the tensor pipe at the clock that the power
+// 159 us, 6.6 TB/s); with several the tensor pipe at the clock that the power
 // limit leaves (817 x 4096 x 151936: 640 us, 448 cycles a K slice of 224
-// columns, the products' own time, at 1.44 GHz).  With hidden rows as the N
-// operand 817 rows pad to 896 columns of four tiles that use every SM, and a
-// few rows to 32 instead of a 128-row operand; pairing halves each SM's share
-// of the hidden tile, so the ring holds 7 to 12 slices.  Before (one SM per 128
-// hidden rows x 256 ids, 4 slices): 192 us and 684 us at these shapes, 28.1
-// instead of 12.3 us for 9 x 1024 x 32000 (its reduction over the ranges was a
-// serial loop per row), 103 instead of 90 for 257 x 2048 x 100001.
+// columns, the products' own time, at 1.44 GHz; the pipe is 94 % busy in an
+// isolated launch of 583 us).  With hidden rows as the N operand 817 rows pad to
+// 896 columns of four tiles that use every SM, and a few rows to 32 instead of a
+// 128-row operand; pairing halves each SM's share of the hidden tile, so the
+// ring holds 7 to 12 slices.  Before (one SM per 128 hidden rows x 256 ids, 4
+// slices): 192 us and 684 us at these shapes, 28.1 instead of 11.5 us for 9 x
+// 1024 x 32000 (its reduction over the ranges was a serial loop per row), 103
+// instead of 86 for 257 x 2048 x 100001.  The epilogue's maxima are float redux
+// instructions: with integer keys made of the values it outlasted the products
+// at short K (1000 x 1024 x 33000 45.8 us, now 39.0).
 #include <cudaTypedefs.h>
 #include <limits.h>
 
@@ -68,7 +71,6 @@ constexpr int kOffAbort = kOffTmemSlot + 4;
 constexpr int kOffRing = 1024;     // stages start 1024-byte aligned
 constexpr int kSmemMax = 232448 - 1024;  // less the room to align the base
 static_assert(kOffAbort + 4 <= kOffRing, "barriers fit below the ring");
-constexpr uint32_t kKeyNegInf = 0x007fffffu;  // order key of -inf
 
 constexpr int stage_bytes(int nt) { return kABytes + nt / 2 * BK * 2; }
 constexpr int stages_of(int nt) {
@@ -81,17 +83,16 @@ struct LmArgs {
   int nt, n_tiles;          // hidden rows per tile, tiles
   int groups, v_tiles;      // vocab ranges, 256-id vocab tiles
   int stages;
-  uint32_t* part_key;       // [groups][M] order keys of the maxima
+  float* part_val;          // [groups][M] maxima
   int32_t* part_idx;        // [groups][M]
   int* err;
 };
 
-// Order-preserving unsigned key of a float (both zeros map to one key); 0
-// stands for a NaN.
-__device__ __forceinline__ uint32_t order_key(float x) {
-  const uint32_t b = __float_as_uint(x + 0.f);
-  if (x != x) return 0u;
-  return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+// The warp's maximum (NaNs passed over), in every lane: one instruction.
+__device__ __forceinline__ float warp_max(float x) {
+  float m;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -301,11 +302,11 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
     // ---------------------------------------------------------------- epilogue
     const int q = warp & 3;            // TMEM lane quarter this warp may access
     const int half = (warp - 2) >> 2;  // takes the 32-column chunks of this parity
-    uint32_t best[BN / 64];            // this lane's column of each chunk: running maximum (order key)
+    float best[BN / 64];               // this lane's column of each chunk: running maximum
     int bi[BN / 64];
 #pragma unroll
     for (int j = 0; j < BN / 64; ++j) {
-      best[j] = kKeyNegInf;
+      best[j] = -INFINITY;
       bi[j] = -1;
     }
     bool ok = true;
@@ -316,7 +317,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
       if (!ok) break;
       tc_fence_after();
       const int v0 = (2 * (t_lo + t) + rank) * BV + q * 32;  // id of the warp's first lane
-      const bool in = v0 + lane < A.V;
+      const bool full = v0 + 32 <= A.V;
 #pragma unroll
       for (int j = 0; j < BN / 64; ++j) {
         const int c = 2 * j + half;
@@ -324,21 +325,26 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
           uint32_t r[32];
           tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + a * BN + c * 32, r);
           tmem_wait_ld();
-          uint32_t mk = 0u;
-          int ml = 0;
+          if (!full) {  // the vocabulary ends inside the warp's ids
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (v0 + lane >= A.V) r[i] = 0xff800000u;  // -inf
+          }
+          float mx = -INFINITY;  // this lane's column: its maximum and the lanes that hold it
+          uint32_t who = 0u;
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            const uint32_t key = in ? order_key(__uint_as_float(r[i])) : 0u;
-            const uint32_t m = __reduce_max_sync(0xffffffffu, key);
-            const uint32_t who = __ballot_sync(0xffffffffu, key == m);
+            const float x = __uint_as_float(r[i]);
+            const float m = warp_max(x);
+            const uint32_t eq = __ballot_sync(0xffffffffu, x == m);
             if (lane == i) {
-              mk = m;
-              ml = __ffs(who) - 1;
+              mx = m;
+              who = eq;
             }
           }
-          if (mk > best[j]) {
-            best[j] = mk;
-            bi[j] = v0 + ml;
+          if (mx > best[j]) {  // (a NaN or -inf never is)
+            best[j] = mx;
+            bi[j] = v0 + __ffs(who) - 1;
           }
         }
       }
@@ -348,14 +354,14 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
     }
     // the pair's maxima meet in the first CTA's ring, which nothing writes or
     // reads any more once the last accumulator is complete: [8 quarters][256]
-    // keys, then ids
+    // maxima, then ids
     if (ok) {
       const uint32_t base = in_first_cta(sb + kOffRing) + (rank * 4 + q) * BN * 4;
 #pragma unroll
       for (int j = 0; j < BN / 64; ++j) {
         const int c = 2 * j + half;
         if (c * 32 < A.nt) {
-          st_cluster(base + (c * 32 + lane) * 4, best[j]);
+          st_cluster(base + (c * 32 + lane) * 4, __float_as_uint(best[j]));
           st_cluster(base + 8 * BN * 4 + (c * 32 + lane) * 4, (uint32_t)bi[j]);
         }
       }
@@ -367,19 +373,20 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
   __syncthreads();
   cluster_sync();
   if (rank == 0 && !*abort_flag && (int)threadIdx.x < A.nt && n0 + (int)threadIdx.x < A.M) {
-    const uint32_t* keys = reinterpret_cast<const uint32_t*>(smem + kOffRing) + threadIdx.x;
-    const int* ids = reinterpret_cast<const int*>(keys) + 8 * BN;
-    uint32_t bk = 0u;
+    const float* vals = reinterpret_cast<const float*>(smem + kOffRing) + threadIdx.x;
+    const int* ids = reinterpret_cast<const int*>(vals) + 8 * BN;
+    float best = -INFINITY;
     int b = -1;
+#pragma unroll
     for (int p = 0; p < 8; ++p) {
-      const uint32_t k = keys[p * BN];
+      const float v = vals[p * BN];
       const int i = ids[p * BN];
-      if (i >= 0 && (b < 0 || k > bk || (k == bk && i < b))) {
-        bk = k;
+      if (i >= 0 && (v > best || (v == best && i < b))) {
+        best = v;
         b = i;
       }
     }
-    A.part_key[(int64_t)g * A.M + n0 + threadIdx.x] = bk;
+    A.part_val[(int64_t)g * A.M + n0 + threadIdx.x] = best;
     A.part_idx[(int64_t)g * A.M + n0 + threadIdx.x] = b;
   }
   if (warp == 1) {
@@ -390,23 +397,23 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
 
 // The first maximum over the vocab ranges, a warp per row.
 __global__ void __launch_bounds__(256)
-lm_head_reduce_kernel(const uint32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx, int groups, int M,
+lm_head_reduce_kernel(const float* __restrict__ part_val, const int32_t* __restrict__ part_idx, int groups, int M,
                       int32_t* __restrict__ out, const int32_t* __restrict__ out_index) {
   pdl_begin();
   const int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (r >= M) return;
-  uint32_t bk = 0u;  // a range without an id leaves 0, below every value's key
+  float best = -INFINITY;
   int b = INT_MAX;
   for (int g = lane; g < groups; g += 32) {
-    const int i = part_idx[(int64_t)g * M + r];
-    const uint32_t k = i >= 0 ? part_key[(int64_t)g * M + r] : 0u;
-    if (k > bk) {  // ranges come in id order
-      bk = k;
+    const int i = part_idx[(int64_t)g * M + r];  // -1: no logit of the range was above -inf
+    const float v = part_val[(int64_t)g * M + r];
+    if (i >= 0 && v > best) {  // ranges come in id order
+      best = v;
       b = i;
     }
   }
-  const uint32_t m = __reduce_max_sync(0xffffffffu, bk);
-  const int id = __reduce_min_sync(0xffffffffu, bk == m ? b : INT_MAX);
+  const float m = warp_max(best);
+  const int id = __reduce_min_sync(0xffffffffu, best == m ? b : INT_MAX);
   if (lane == 0) out[out_index ? out_index[r] : r] = id == INT_MAX ? 0 : id;
 }
 
@@ -466,7 +473,7 @@ LmPlan plan_lm_head(int rows, int vocab) {
       p.groups = groups;
     }
   }
-  p.ws_bytes = ((size_t)p.groups * rows * (sizeof(uint32_t) + sizeof(int32_t)) + 255) / 256 * 256;
+  p.ws_bytes = ((size_t)p.groups * rows * (sizeof(float) + sizeof(int32_t)) + 255) / 256 * 256;
   return p;
 }
 
@@ -496,13 +503,13 @@ cudaError_t launch_lm_head_argmax(const LmPlan& p, const uint16_t* hidden, const
   a.groups = p.groups;
   a.v_tiles = p.v_tiles;
   a.stages = stages_of(p.nt);
-  a.part_key = static_cast<uint32_t*>(workspace);
-  a.part_idx = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)p.groups * rows * sizeof(uint32_t));
+  a.part_val = static_cast<float*>(workspace);
+  a.part_idx = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)p.groups * rows * sizeof(float));
   a.err = err;
   e = launch_pdl(lm_head_argmax_kernel, dim3(2 * p.n_tiles * p.groups), dim3(kThreads),
                  1024 + kOffRing + a.stages * stage_bytes(p.nt), s, mh, mw, a);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(lm_head_reduce_kernel, dim3((rows + 7) / 8), dim3(256), 0, s, a.part_key, a.part_idx, p.groups,
+  e = launch_pdl(lm_head_reduce_kernel, dim3((rows + 7) / 8), dim3(256), 0, s, a.part_val, a.part_idx, p.groups,
                  rows, out, out_index);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
