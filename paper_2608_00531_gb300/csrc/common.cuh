@@ -83,11 +83,13 @@ cudaError_t launch_build_tree(const cure_tree_params& p, const int32_t* top_ids,
                               uint64_t* anc, int32_t* ufp_pos, int32_t* n_ufp, int* err,
                               cudaStream_t s);
 
+// after_argmax: launched right after launch_target_argmax on the same stream.
 cudaError_t launch_accept_walk(int batch, int n_max, int block, const int32_t* n_nodes,
                                const int32_t* tok, const int32_t* parent, const int32_t* depth,
                                const uint64_t* anc, const int32_t* targ, int32_t* accept_len,
                                int32_t* best_node, int32_t* path_nodes, int32_t* out_tokens,
-                               int32_t* diverge_depth, int* err, cudaStream_t s);
+                               int32_t* diverge_depth, bool after_argmax, int* err,
+                               cudaStream_t s);
 
 struct LayerPtrs {
   void* k[kMaxLayers];

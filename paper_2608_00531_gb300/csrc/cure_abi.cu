@@ -302,7 +302,7 @@ cure_status cure_accept(const void* target_logits, int32_t* targ, int32_t batch,
   }
   return from_cuda(launch_accept_walk(batch, n_max, block, n_nodes, tok, parent, depth, anc, targ,
                                       accept_len, best_node, path_nodes, out_tokens, diverge_depth,
-                                      err, s));
+                                      target_logits != nullptr, err, s));
 }
 
 cure_status cure_resync_kv(int32_t layers, void* const* k_caches, void* const* v_caches,

@@ -125,8 +125,7 @@ struct TopK {
 
 // Base-2 log-sum-exp state: sum of 2^(x*log2e - mb).
 struct Lse2 {
-  float m;   // natural-log running max (for the rescale test)
-  float mb;  // m * log2e as used in the exponents
+  float mb;  // base: the running max * log2e, as used in the exponents
   float s;
 };
 
@@ -539,7 +538,7 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
   WarpTop<KT> tk;   // the warp's list
   ll.init();
   tk.init();
-  Lse2 ls{-INFINITY, -INFINITY, 0.f};
+  Lse2 ls{-INFINITY, 0.f};
   if (c == 0 && warp == 0 && a0 > 0) {  // the ids before the first 16-byte boundary
     const float x = lane < a0 ? bf16_lo(rowp[lane]) : 0.f;
     if (lane < a0) lse_add(ls, x);
