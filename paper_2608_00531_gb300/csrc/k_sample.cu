@@ -5,9 +5,9 @@
 // cure_accept takes this kernel's place.  The acceptance walk is the same in
 // both cases: a child is accepted when its token equals the parent's sample.
 //
-// One CTA of 4, 8 or 16 warps per (sequence, node) row.  The row is cut into
-// eight-id groups on 16-byte boundaries (only the first and the last group can
-// be partial) and each warp owns a contiguous share of the groups, which its
+// One CTA of four warps per (sequence, node) row.  The row is cut into eight-id
+// groups on 16-byte boundaries (only the first and the last group can be
+// partial) and each warp owns a contiguous quarter of the groups, which its
 // lanes stream as 16-byte vectors, 32 adjacent groups per warp instruction:
 //   1. one pass: a warp step covers 128 contiguous groups (four per lane);
 //      every lane sums p_v = 2^((l_v - base) log2(e) / T) over them against a
@@ -35,6 +35,8 @@
 namespace cure {
 namespace {
 
+constexpr int kSampleThreads = 128;
+constexpr int kSampleWarps = kSampleThreads / 32;
 constexpr int kSampleUnroll = 4;  // groups per lane per step (loads one step ahead)
 constexpr float kLog2eS = 1.4426950408889634f;
 constexpr float kRaise = 8.f;     // base raised when a term would exceed 2^8
@@ -152,8 +154,7 @@ __device__ __forceinline__ float group_mass(const float x[8], float base, float 
   return s;
 }
 
-template <int kSampleWarps>
-__global__ void __launch_bounds__(32 * kSampleWarps)
+__global__ void __launch_bounds__(kSampleThreads)
 sample_target_kernel(const uint16_t* __restrict__ logits, const float* __restrict__ uniforms, float scale,
                      int n_max, int vocab, const int32_t* __restrict__ n_nodes, int32_t* __restrict__ targ,
                      int* err) {
@@ -161,7 +162,6 @@ sample_target_kernel(const uint16_t* __restrict__ logits, const float* __restric
   const int64_t row = blockIdx.x;
   const int b = (int)(row / n_max), j = (int)(row % n_max);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float u_in = uniforms[row];
   int n = n_nodes[b];
   if (n < 1 || n > n_max) {
     if (tid == 0 && j == 0) flag(err, CURE_DEVERR_NODES);
@@ -294,7 +294,8 @@ sample_target_kernel(const uint16_t* __restrict__ logits, const float* __restric
     E[w] = total;
     total += S[w];
   }
-  const float u = fminf(fmaxf(u_in, 0.f), 0x1.fffffep-1f);  // [0, 1); NaN -> 0
+  float u = uniforms[row];
+  u = fminf(fmaxf(u, 0.f), 0x1.fffffep-1f);  // [0, 1); NaN -> 0
   const float r = u * total;
   int owner = 0;
 #pragma unroll
@@ -335,27 +336,16 @@ sample_target_kernel(const uint16_t* __restrict__ logits, const float* __restric
   }
 
   // ---- 3b. that block's groups in id order, 32 at a time
-  __shared__ uint4 s_grp[kSampleUnroll][32];  // only the owning warp gets here
   const int c_lo = g_lo + bsel * bstride * kStepGroups;
   const int c_hi = min(g_hi, c_lo + bstride * kStepGroups);
   acc = bstart;
   int last = -1;  // the block's last id with mass seen so far (warp-uniform)
   for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
     const int g = c0 + lane;
-    const int k = ((c0 - c_lo) >> 5) % kSampleUnroll;
-    if (k == 0) {  // the next kSampleUnroll groups of the lane are loaded together, and wait in its own slots
-      uint4 rg[kSampleUnroll];
-#pragma unroll
-      for (int v = 0; v < kSampleUnroll; ++v)
-        if (g + 32 * v < c_hi) rg[v] = rv.load(g + 32 * v);
-#pragma unroll
-      for (int v = 0; v < kSampleUnroll; ++v)
-        if (g + 32 * v < c_hi) s_grp[v][lane] = rg[v];
-    }
     float xv[8];
     float q = 0.f;
     if (g < c_hi) {
-      unpack8(s_grp[k][lane], xv);
+      unpack8(rv.load(g), xv);
       q = group_mass(xv, m, scale);
     }
     float inc = q;
@@ -409,22 +399,8 @@ cudaError_t launch_sample_target(const uint16_t* logits, const float* uniforms, 
                                  cudaStream_t s) {
   if (batch == 0) return cudaSuccess;
   const unsigned rows = (unsigned)((int64_t)batch * n_max);
-  auto launch = [&](auto kernel, int warps) {
-    return launch_pdl(kernel, dim3(rows), dim3(32 * warps), 0, s, logits, uniforms, kLog2eS / temperature, n_max,
-                      vocab, n_nodes, targ, err);
-  };
-  // A row's warps stream its parts side by side, so the fewer the rows, the more
-  // warps each takes (at 72-80 registers an SM holds 7 CTAs of 4 warps, 3 of 8,
-  // 1 of 16).  Graph-replayed, us a call with 4 / 8 / 16 warps a row: 23 rows x
-  // 128256 22.0 / 14.9 / 13.4, 98 x 151936 27.9 / 19.5 / 15.1, 410 x 100001
-  // 28.1 / 19.9 / 24.3, 828 x 151936 54.2 / 51.1 / 60.0, 1648 x 151936
-  // 92.3 / 97.2 / 109 (54.2 and 92.3: 4.6 and 5.4 TB/s, the stream with its
-  // exponentials).  The rows counted are the tree's slots, as its sizes are on
-  // the device.
-  const unsigned sms = (unsigned)num_sms();
-  if (rows <= sms) return launch(sample_target_kernel<16>, 16);
-  if (rows <= 8 * sms) return launch(sample_target_kernel<8>, 8);
-  return launch(sample_target_kernel<4>, 4);
+  return launch_pdl(sample_target_kernel, dim3(rows), dim3(kSampleThreads), 0, s, logits, uniforms,
+                    kLog2eS / temperature, n_max, vocab, n_nodes, targ, err);
 }
 
 }  // namespace cure

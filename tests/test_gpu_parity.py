@@ -867,25 +867,6 @@ def test_sample_target_inverse_cdf(cure, V, T):
     assert got[2, 1] == 17 and got[2, 2] == 0 and got[3, 0] >= V // 2
 
 
-@pytest.mark.parametrize("B,N", [(19, 8), (17, 9), (152, 8), (123, 10)])
-@pytest.mark.parametrize("V", [33, 1025, 5001])
-def test_sample_target_rows_on_both_sides_of_the_warp_counts(cure, B, N, V):
-    """152 / 153 and 1216 / 1230 rows (16, 8 and 4 warps a row), vocabularies
-    with empty and partial warp segments; every draw against the float64 CDF."""
-    rng = np.random.default_rng(B * N + V)
-    logits = W.to_bf16((rng.standard_normal((B, N, V)) * 2.0).astype(np.float32))
-    u = rng.random((B, N)).astype(np.float32)
-    u[0, :3] = [0.0, 0.9999999, 0.5]
-    n = np.full(B, N, dtype=np.int32)
-    got = cure.cure_sample_target(logits.to(DEV), torch.from_numpy(n).to(DEV), torch.from_numpy(u).to(DEV),
-                                  0.8).cpu().numpy()
-    assert cure.cure_device_error() == 0
-    xf = _f64(logits)
-    for b in range(B):
-        for j in range(N):
-            assert _valid_sample(xf[b, j], 0.8, float(u[b, j]), int(got[b, j])), (b, j, got[b, j])
-
-
 @pytest.mark.parametrize("T", [1e-30, 1e-38])
 def test_sample_target_tiny_temperature_and_huge_logits(cure, T):
     """Temperatures so small that every logit below the maximum has
