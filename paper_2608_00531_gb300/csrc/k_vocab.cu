@@ -213,37 +213,6 @@ template <int KT>
 struct WarpTop {
   uint32_t key[KT];
   int id[KT];
-  __device__ __forceinline__ void init() {
-#pragma unroll
-    for (int k = 0; k < KT; ++k) {
-      key[k] = 0u;
-      id[k] = INT_MAX;
-    }
-  }
-  // (x, ix) goes in behind every entry at or above it: the caller offers equal
-  // values in id order.
-  __device__ __forceinline__ void insert(uint32_t x, int ix) {
-#pragma unroll
-    for (int k = KT - 1; k > 0; --k) {
-      const bool here = x > key[k], above = x > key[k - 1];
-      key[k] = above ? key[k - 1] : here ? x : key[k];
-      id[k] = above ? id[k - 1] : here ? ix : id[k];
-    }
-    if (x > key[0]) {
-      key[0] = x;
-      id[0] = ix;
-    }
-  }
-  // Takes one candidate per lane (key 0: none), best first, lowest id on ties.
-  __device__ __forceinline__ void offer(uint32_t x, int ix) {
-    while (true) {
-      const uint32_t best = __reduce_max_sync(0xffffffffu, x);
-      if (best <= key[KT - 1]) break;
-      const int i = __reduce_min_sync(0xffffffffu, x == best ? ix : INT_MAX);
-      insert(best, i);
-      if (x == best && ix == i) x = 0u;
-    }
-  }
 };
 
 // The warp's list from the lanes' sorted lists: round k takes the best head
@@ -472,14 +441,14 @@ vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int n_max, con
 // so that fewer logits enter a list; every warp writes its result straight
 // into rank 0's shared memory, one cluster barrier follows, and one warp
 // merges all parts at once (before: a merge per CTA, two barriers, and a
-// serial walk over the peers' shared memory by one thread).  Up to top-4 each
-// lane keeps its own list (several logits enter at once, and the code for the
-// inserts stays small: top-3 of 512 x 151936 30.4 us against 37.3 with one
-// list per warp); above, the warp keeps one list, entered one logit at a
-// time, since a lane's 24 unrolled inserts of an 8-deep list no longer fit
-// the instruction cache (top-6 of 512 x 151936: 65 us against 133).
+// serial walk over the peers' shared memory by one thread).  Each lane keeps its
+// own list, so that several logits enter at once.  Up to top-4 the 24 inserts of
+// a step are unrolled; above, a lane loops over a mask of its candidates, since
+// 24 unrolled inserts of an 8-deep list do not fit the instruction cache (top-6
+// of 512 x 151936: 44.8 us; unrolled 133; one list per warp, entered one logit
+// at a time, 65).
 // Before these changes and the launch shapes of pick_scan: 512 x 151936 top-3
-// 36.7 us, top-6 306 us, 16 x 128256 12.0 us, 128 x 151936 33.6 us (now 14).
+// 36.7 us, top-6 306 us (now 44.8), 16 x 128256 12.0 us, 128 x 151936 33.6 us (now 14).
 //
 // Vectors per lane per step: three 16-byte loads in flight per lane (70
 // registers up to top-3, still one wave of the grid).
@@ -533,34 +502,26 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
     if (vi < ve) r[u] = ld_stream(vp + vi);
   }
 
-  constexpr bool kLaneLists = KT <= 4;
-  TopK<KT> ll;      // lane lists, or
-  WarpTop<KT> tk;   // the warp's list
+  TopK<KT> ll;
   ll.init();
-  tk.init();
   Lse2 ls{-INFINITY, 0.f};
   if (c == 0 && warp == 0 && a0 > 0) {  // the ids before the first 16-byte boundary
     const float x = lane < a0 ? bf16_lo(rowp[lane]) : 0.f;
     if (lane < a0) lse_add(ls, x);
-    if constexpr (kLaneLists) {
-      if (lane < a0) ll.insert(x, lane);
-    } else {
-      tk.offer(lane < a0 ? order_key(x) : 0u, lane);
-    }
+    if (lane < a0) ll.insert(x, lane);
   }
 
-  // The trip count is uniform over the warp: the list, the threshold and the
-  // log-sum-exp base are warp-wide values that all lanes take part in.
-  //  - tkey: the least order key that can still enter the list: above the
-  //    warp's own k-th best (an equal one comes later in id order), and at or
-  //    above the largest k-th best of the CTA's warps so far (a warp publishes
-  //    its own after each change, and reads the CTA's best once a step).  So
-  //    lists change only in rare steps.
+  // The trip count is uniform over the warp: the threshold and the log-sum-exp
+  // base are warp-wide values that all lanes take part in.
+  //  - tkey: the order key of a lower bound on the row's k-th best: the largest
+  //    bound of the CTA's warps so far (a warp publishes its own when its lists
+  //    change, and reads the CTA's best once a step).  A logit below it cannot
+  //    be in the row's top k, so lists change only in rare steps.
   //  - mbw: base-2 exponent base of the lane sums (sum of 2^(x log2e - mbw));
   //    raised, with the sums rescaled, only when some lane sees a logit more
   //    than 2^8 above it, so the sums stay below 2^8 per term and the rescale
   //    is rare and uniform.
-  uint32_t tkey = kLaneLists ? 0u : tk.key[KT - 1] + 1u;
+  uint32_t tkey = 0u;
   float mbw = -INFINITY;
   uint64_t sacc = f2_pack(0.f, 0.f);  // two lane sums, as one f32x2 pair
   // one step: kUnrollS vectors per lane; FULL when every lane's vectors are in
@@ -614,21 +575,21 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
       }
     }
     tkey = max(tkey, *reinterpret_cast<volatile uint32_t*>(&thr_s));
-    if constexpr (kLaneLists) {
-      if (wb == wb0) {
-        // first step: the k-th largest of the lanes' maxima of this step is a
-        // valid threshold already, so that a warp does not start by inserting
-        // every logit it sees
-        float gm = gl;
+    if (wb == wb0) {
+      // first step: the k-th largest of the lanes' maxima of this step is a
+      // valid threshold already, so that a warp does not start by inserting
+      // every logit it sees
+      float gm = gl;
 #pragma unroll
-        for (int k = 0; k < KT; ++k) {
-          const uint32_t mk = __reduce_max_sync(0xffffffffu, order_key(gm));
-          if (k == KT - 1) tkey = max(tkey, mk);
-          if (gm == key_value(mk)) gm = -INFINITY;
-        }
+      for (int k = 0; k < KT; ++k) {
+        const uint32_t mk = __reduce_max_sync(0xffffffffu, order_key(gm));
+        if (k == KT - 1) tkey = max(tkey, mk);
+        if (gm == key_value(mk)) gm = -INFINITY;
       }
-      const float thr = key_value(tkey);
-      if (__any_sync(0xffffffffu, gl >= thr)) {
+    }
+    const float thr = key_value(tkey);
+    if (__any_sync(0xffffffffu, gl >= thr)) {
+      if constexpr (KT <= 4) {
 #pragma unroll
         for (int u = 0; u < kUnrollS; ++u) {
           if ((FULL || wb + lane + u * T < ve) && gmv[u] >= thr) {
@@ -642,57 +603,36 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
             }
           }
         }
-        tkey = max(tkey, warp_kth_key(ll));
-        if (lane == 0) atomicMax(&thr_s, tkey);
-      }
-    } else if (__any_sync(0xffffffffu, gl >= key_value(tkey))) {
-      // the step's best logits enter one at a time, lowest id on ties; one
-      // that has entered is blanked out as a NaN, which the maxima pass over
-      uint32_t lk = FULL || wb + lane < ve ? order_key(gl) : 0u;
-      while (true) {
-        const uint32_t best = __reduce_max_sync(0xffffffffu, lk);
-        if (best < tkey) break;
-        int at = INT_MAX;  // this lane's first logit equal to it
-        if (lk == best) {
-          const float v = key_value(best);
+      } else {
+        uint32_t cand = 0u;  // this lane's logits at or above it, in id order
 #pragma unroll
-          for (int u = kUnrollS - 1; u >= 0; --u) {
-            if (FULL || wb + lane + u * T < ve) {
-              const uint32_t w[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
+        for (int u = 0; u < kUnrollS; ++u) {
 #pragma unroll
-              for (int q = 3; q >= 0; --q) {
-                if (bf16_hi(w[q]) == v) at = u * T * 8 + 2 * q + 1;
-                if (bf16_lo(w[q]) == v) at = u * T * 8 + 2 * q;
-              }
-            }
+          for (int q = 0; q < 4; ++q) {
+            float a, b;
+            f2_unpack(xp[u][q], a, b);
+            const bool in = FULL || wb + lane + u * T < ve;
+            if (in && a >= thr) cand |= 1u << (8 * u + 2 * q);
+            if (in && b >= thr) cand |= 2u << (8 * u + 2 * q);
           }
         }
-        const int id0 = a0 + ((wb + lane) << 3);
-        const int id = __reduce_min_sync(0xffffffffu, at == INT_MAX ? INT_MAX : id0 + at);
-        tk.insert(best, id);
-        tkey = max(tkey, tk.key[KT - 1] + 1u);
-        if (at != INT_MAX && id0 + at == id) {
-          float g = -INFINITY;
-          bool left = false;
+#pragma unroll 1
+        while (cand) {
+          const int e = __ffs(cand) - 1;
+          cand &= cand - 1u;
+          uint32_t w = 0u;  // the word of logit e (masks, not an indexed array)
 #pragma unroll
           for (int u = 0; u < kUnrollS; ++u) {
-            if (FULL || wb + lane + u * T < ve) {
-              uint32_t w[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
+            const uint32_t wu[4] = {r[u].x, r[u].y, r[u].z, r[u].w};
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                if (at == u * T * 8 + 2 * q) w[q] |= 0x00007fffu;
-                if (at == u * T * 8 + 2 * q + 1) w[q] |= 0x7fff0000u;
-                const float lo = bf16_lo(w[q]), hi = bf16_hi(w[q]);
-                g = fmaxf(g, fmaxf(lo, hi));
-                left |= lo == lo || hi == hi;
-              }
-              r[u] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+            for (int q = 0; q < 4; ++q) w |= wu[q] & (0u - (uint32_t)((e >> 1) == 4 * u + q));
           }
-          lk = left ? order_key(g) : 0u;
+          ll.insert((e & 1) ? bf16_hi(w) : bf16_lo(w), a0 + ((wb + lane + (e >> 3) * T) << 3) + (e & 7));
         }
+        __syncwarp();
       }
-      if (lane == 0) atomicMax(&thr_s, tk.key[KT - 1]);
+      tkey = max(tkey, warp_kth_key(ll));
+      if (lane == 0) atomicMax(&thr_s, tkey);
     }
 #pragma unroll
     for (int u = 0; u < kUnrollS; ++u) r[u] = nx[u];
@@ -707,13 +647,10 @@ vocab_scan_kernel(const uint16_t* __restrict__ logits, int vocab, int k_out,
     const int i = tail0 + lane;
     const float x = i < vocab ? bf16_lo(rowp[i]) : 0.f;
     if (i < vocab) lse_add(ls, x);
-    if constexpr (kLaneLists) {
-      if (i < vocab) ll.insert(x, i);
-    } else {
-      tk.offer(i < vocab ? order_key(x) : 0u, i);
-    }
+    if (i < vocab) ll.insert(x, i);
   }
-  if constexpr (kLaneLists) warp_merge(ll, tk);
+  WarpTop<KT> tk;
+  warp_merge(ll, tk);
 
   // ---- every warp's result goes to rank 0's shared memory
   warp_lse(ls);
