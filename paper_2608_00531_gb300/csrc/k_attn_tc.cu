@@ -731,6 +731,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       for (int j = 0; ok && j < n; ++j) {
         const uint32_t gt = gk0 + (uint32_t)j;
         if (sc > 0 && !wait_warp(bar(B_SFREE + m), (sc - 1) & 1u, abort_flag, A.err)) { ok = false; break; }
+        // A parity wait is only sound one phase behind.  This issuer has not waited
+        // for the K tiles of the other slot's pieces, so the stage's previous tile
+        // may still be in flight; it has landed once its PV product is done, which
+        // the producer waits for before it loads this tile.  (That barrier cannot
+        // run ahead: tile gt's own PV product needs this S.)
+        if (PINGPONG && gt >= NS && !wait_warp(bar(B_KVEMPTY + gt % NS), ((gt / NS) & 1u) ^ 1u, abort_flag, A.err)) {
+          ok = false;
+          break;
+        }
         if (!wait_warp(bar(B_KFULL + gt % NS), (gt / NS) & 1u, abort_flag, A.err)) { ok = false; break; }
         tc_fence_after();
         // a paged cache tile interleaves the d halves per 8-key group

@@ -482,6 +482,30 @@ def test_tree_attn_many_one_tile_units(cure, Hq, Hkv, paged, in_place):
         _cmp_attn(got, ref, t)
 
 
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("paged", [False, True])
+def test_tree_attn_short_pieces_before_long_ones(cure, paged, in_place):
+    """Units of 1 to 4 tiles alternate with units of 11, so that CTA ranges
+    begin with a piece shorter than the K/V ring and go on with one that goes
+    round it: the second slot's products start on stages whose first tiles it
+    never waited for."""
+    B, Hq, Hkv = 240, 4, 1
+    lens = [(640, 50, 620, 100, 650, 170, 600, 3)[i % 8] for i in range(B)]
+    if in_place:
+        t, q, kc, vc, L, table, npages = _in_place_case(B, 12, 8, Hq, Hkv, lens, paged, seed=11)
+        tk = tv = None
+    else:
+        t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 12, 8, Hq, Hkv, lens, paged, 1.0, 1.0, seed=11)
+    ref = oracle.tree_attn(_f64(q), None if tk is None else _f64(tk), None if tv is None else _f64(tv), _f64(kc),
+                           _f64(vc), L, t["n_nodes"], t["anc"], 1.0 / math.sqrt(128), table, 16)
+    for _ in range(3):
+        if in_place:
+            got = _run_attn_in_place(cure, t, q, kc, vc, L, table, npages, Hkv)
+        else:
+            got = _run_attn(cure, t, q, tk, tv, kc, vc, L, table, npages, Hkv)
+        _cmp_attn(got, ref, t)
+
+
 @pytest.mark.parametrize("paged", [False, True])
 def test_tree_attn_split_units_on_garbage_workspace(cure, paged):
     """96 units, too many for a cluster each: the units cut by the stream-K
