@@ -675,16 +675,19 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         issue_k(sb + kOffK + st * kTile, bar(B_KFULL + st));
         __syncwarp();
         ++k_issued;
-        // a cluster's CTA has one piece, and a ping-pong piece's Q slot is long
-        // free: Q goes between the first K and V
-        if (MODE != kStreamK && t == s.t0 && !load_q()) { ok = false; break; }
+        // a cluster's CTA has one piece and nothing else to do: Q goes between the
+        // first K and V.  In the other modes it goes after V, which the products of
+        // the pieces before are queued up for (ping-pong with Q in between: 30
+        // sequences x 8 kv heads of 1 query head, 200-6000 keys 77.1 us, now 70.0;
+        // 60 x 16 of 1, 1000-2000 keys 150.8, now 142.3)
+        if (MODE == kCluster && t == s.t0 && !load_q()) { ok = false; break; }
         if (lane == 0) mbar_arrive_expect_tx(bar(B_VFULL + st), kTile);
         __syncwarp();
         issue_v(sb + kOffV + st * kTile, bar(B_VFULL + st));
         __syncwarp();
         ++v_issued;
         ++gk;
-        if (MODE == kStreamK && t == s.t0 && !load_q()) { ok = false; break; }
+        if (MODE != kCluster && t == s.t0 && !load_q()) { ok = false; break; }
       }
     }
     if (*abort_flag) {  // let copies in flight land before the CTA's smem goes away
@@ -1456,10 +1459,15 @@ cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;
   // Ping-pong where every unit fits one M tile and a CTA has at least 1.5 units
-  // on average: it hides the pieces' starts and ends (64 sequences x 8 kv heads x
-  // 200-300 keys 46.6 -> 39.9 us, 16 x 16 x 500-900 36.4 -> 33.0, 32 x 8 x 1024-8192
-  // 111.8 -> 108.6), and with fewer, longer pieces its tiles cost 1 % more (16 x 8 x
-  // 1024-8192, 0.84 units a CTA, 61.5 -> 62.2; 20 x 8 x 3000-9000, 1.05, 84.9 -> 86.2).
+  // on average: it hides the pieces' starts and ends.  us per call, stream-K ->
+  // ping-pong (sequences x kv heads of query heads, keys; units a CTA):
+  //   64 x 8 of 4, 200-300 (3.4)        47.0 -> 41.0
+  //   16 x 16 of 1, 500-900 (1.7)       36.6 -> 34.2
+  //   60 x 16 of 1, 1000-2000 (6.3)    144.5 -> 143.0
+  //   32 x 8 of 4, 1024-8192 (1.7)     113.3 -> 108.2
+  //   15 x 16 of 1, 32768 (1.6)          651 -> 631
+  // With fewer pieces there is little to hide: 16 x 8 of 4, 1024-8192 (0.84) 62.2 ->
+  // 62.4; 20 x 8 of 5, 3000-9000 (1.05) 87.7 -> 87.9.
   const bool one_tile = A.n_max <= BM / A.G;
   const int mode = A.cluster > 0 ? kCluster : one_tile && 2 * (int64_t)A.units_max >= 3 * (int64_t)grid.x ? kPingPong : kStreamK;
   e = cudaLaunchKernelEx(&cfg, kKernels[mode][A.inplace ? 1 : 0], mk, mv, mtk, mtv, mq, a);
