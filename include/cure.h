@@ -160,7 +160,8 @@ cure_status cure_build_tree(const cure_tree_params* p, const int32_t* top_ids, c
  * verifies every tree path in one pass).  For sequence b, node j < n_nodes[b],
  * query head h (kv head h / (heads_q / heads_kv)):
  *   out[b][j][h] = softmax(scale * q k^T) v over the cached keys 0..L_b-1 and
- *                  the tree keys a with bit a of anc[b][j] set.
+ *                  the tree keys a with bit a of anc[b][j] set (0 where that
+ *                  leaves no key).
  * q, out: bf16 [B][n_max][heads_q][D]; tree_k, tree_v: bf16 [B][n_max][heads_kv][D]
  * (this step's target keys/values of the tree tokens); k_cache, v_cache: one
  * layer in the layout of `kv` (a HOST pointer).

@@ -55,6 +55,7 @@
 // timeout the CTA raises CURE_DEVERR_TIMEOUT, drains and leaves.
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
+#include <float.h>
 
 #include <algorithm>
 #include <atomic>
@@ -203,6 +204,15 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
+// The base-2 log-sum-exp of a row of a piece.  A row that saw no key gets the lowest
+// finite value: its O is 0, so a merge over pieces that all saw none gives 0
+// (-inf would give NaN there).  A NaN stays one.
+__device__ __forceinline__ float row_lse(float m, float l) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(m + log2f(l)), "f"(-FLT_MAX));
   return d;
 }
 
@@ -1020,7 +1030,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
                            __float_as_uint(__uint_as_float(o[4 * i + 2]) * inv),
                            __float_as_uint(__uint_as_float(o[4 * i + 3]) * inv));
           }
-          lse_s[prow] = m_run + log2f(l_run);
+          lse_s[prow] = row_lse(m_run, l_run);
         }
         continue;  // (the one piece)
       }
@@ -1060,7 +1070,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         // and merges with its O read straight from TMEM.  Otherwise it writes
         // its partial, publishes (release fence + counter), and merges if the
         // counter says it came last.  O_m is released after the merge.
-        const float lse_own = m_run + log2f(l_run);
+        const float lse_own = row_lse(m_run, l_run);
         sync_epilogue();
         if (first)
           *last_flag = (!*abort_flag && count_of(ld_acquire(A.cnt + s.u), A.tag) == s.parts - 1) ? 2 : 0;

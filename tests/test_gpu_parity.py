@@ -606,6 +606,42 @@ def test_tree_attn_in_place_two_words(cure, paged):
     _cmp_attn(got, ref, t)
 
 
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("B,Hkv,n", [
+    (2, 2, 20),     # a cluster of CTAs per unit
+    (30, 8, 20),    # many units of one M tile, whole in their CTA
+    (12, 8, 200),   # row groups of several tree tiles, units cut by the stream-K ranges
+])
+def test_tree_attn_rows_that_see_no_key(cure, B, Hkv, n, in_place):
+    """An empty cache and a node without ancestor bits: nothing to attend to,
+    and the row is zero whichever way the call runs; the other rows are as
+    ever.  (build_tree always sets a node's own bit; a caller's tree need not.)"""
+    Hq, N = 4 * Hkv, n + 1
+    rng = np.random.default_rng(B + n)
+    q = W.normal_bf16((B, N, Hq, 128), 1.0, rng)
+    tk, tv = W.normal_bf16((B, N, Hkv, 128), 1.0, rng), W.normal_bf16((B, N, Hkv, 128), 1.0, rng)
+    kc, vc = W.normal_bf16((B, N + 3, Hkv, 128), 1.0, rng), W.normal_bf16((B, N + 3, Hkv, 128), 1.0, rng)
+    if in_place:
+        kc[:, :N], vc[:, :N] = tk, tv
+    words = (N + 63) // 64
+    bits = np.tril(rng.random((B, n, n)) < 0.3) | np.eye(n, dtype=bool)
+    bits[:, 3::7] = False
+    anc = np.zeros((B, N, words), dtype=np.uint64)
+    for a in range(n):
+        anc[:, :n, a >> 6] |= bits[:, :, a].astype(np.uint64) << np.uint64(a & 63)
+    t = dict(n_nodes=np.full(B, n, dtype=np.int32), anc=anc)
+    L = np.zeros(B, dtype=np.int32)
+    got = _run_attn_in_place(cure, t, q, kc, vc, L, None, 0, Hkv) if in_place else \
+        _run_attn(cure, t, q, tk, tv, kc, vc, L, None, 0, Hkv)
+    k, v = _f64(tk)[:, :n], _f64(tv)[:, :n]
+    s = np.einsum("bjhgd,bahd->bhgja", _f64(q)[:, :n].reshape(B, n, Hkv, 4, 128), k) / math.sqrt(128)
+    p = np.where(bits[:, None, None], np.exp(s - s.max(-1, keepdims=True)), 0.0)
+    p /= np.maximum(p.sum(-1, keepdims=True), 1e-300)
+    ref = np.einsum("bhgja,bahd->bjhgd", p, v).reshape(B, n, Hq, 128)
+    assert (got[:, 3:n:7] == 0).all()
+    _cmp_attn(got, ref, t)
+
+
 def test_tree_attn_full_serve_layer_sampled(cure):
     """One layer at the benchmark's serving shape (batch 32, 28/4 heads, paged
     16-token blocks, lengths U[1024, 8192]); the oracle checks 3 sequences."""
