@@ -462,7 +462,11 @@ struct ScanPart {
   float mb, s;
 };
 
-__device__ __forceinline__ void lse_add(Lse2& ls, float x) { lse_merge(ls, x * kLog2e, 1.f); }
+// One of the few ids at the row's ends, outside its whole vectors (a NaN there is
+// passed over).
+__device__ __forceinline__ void lse_add(Lse2& ls, float x) {
+  if (x == x) lse_merge(ls, x * kLog2e, 1.f);
+}
 
 template <int KT, int T>
 __global__ void __launch_bounds__(T)

@@ -124,6 +124,38 @@ def test_score_draft_launch_shapes(cure, rows, V, k):
     assert torch.equal(ids, torch.arange(k, dtype=torch.int32, device=DEV).expand(rows, k))
 
 
+@pytest.mark.parametrize("k", [2, 3, 6])
+@pytest.mark.parametrize("rows,V", [(9, 4099), (64, 30011), (300, 4111), (600, 2050)])
+def test_score_draft_nan_and_infinite_logits(cure, rows, V, k):
+    """A NaN is never a candidate and both infinities rank as values do,
+    wherever they stand; odd vocabularies put the ends of the rows at every
+    misalignment.  A NaN among the ids after the last whole 16 bytes leaves the
+    log-probability to the other logits."""
+    rng = np.random.default_rng(rows + V + k)
+    x = rng.standard_normal((rows, V), dtype=np.float32)
+    x[0::6, rng.choice(V, V // 2, replace=False)] = np.nan
+    x[1::6, :7] = np.nan
+    x[2::6, -1] = np.nan
+    x[3::6, rng.choice(V, 2, replace=False)] = np.inf
+    x[4::6] = np.nan
+    x[4::6, rng.choice(V, k, replace=False)] = -np.inf
+    x[5::6, -2] = np.inf
+    x[5::6, 0] = np.nan
+    x = W.to_bf16(x)
+    ids, vals, margin, logp1 = (t.cpu().numpy().reshape(rows, -1) for t in cure.cure_score_draft(x.to(DEV), k))
+    y = _f64(x)
+    order = np.argsort(-y, axis=1, kind="stable")[:, :k]  # NaNs last
+    assert np.array_equal(ids, order)
+    top = np.take_along_axis(y, order, 1)
+    assert np.array_equal(vals, top.astype(np.float32))
+    with np.errstate(invalid="ignore"):
+        assert np.array_equal(margin[:, 0], (top[:, 0] - top[:, 1]).astype(np.float32), equal_nan=True)
+    for r in range(2, rows, 6):
+        if (r * V + V) % 8:  # the row ends inside 16 bytes
+            want = top[r, 0] - np.log(np.nansum(np.exp(y[r] - top[r, 0]))) - top[r, 0]
+            assert abs(logp1[r, 0] - want) <= LOGP_TOL * max(1.0, abs(want)), r
+
+
 def test_score_draft_full_long_shape_sampled(cure):
     """batch 64 x block 16 x vocab 128256 with top-2: 1024 rows, one CTA per
     row, the launch the long-context configuration takes; 64 sampled rows."""
