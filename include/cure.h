@@ -338,6 +338,16 @@ cure_status cure_device_error(void* stream, int32_t* bits);
  */
 cure_status cure_selftest_wait_timeout(int64_t limit_cycles, void* stream);
 
+/*
+ * Failure-detection self-test: cure_lm_head_argmax with a wait that runs out
+ * after `limit_cycles` cycles (1 .. 2^30) in one CTA (`rank` 0 or 1) of every
+ * pair.  CURE_DEVERR_TIMEOUT is raised; the tokens are not the argmax, but
+ * each is an id of the vocabulary.
+ */
+cure_status cure_selftest_lm_head_timeout(const void* hidden, const void* w_lm, int32_t rows, int32_t d_model,
+                                          int32_t vocab, int32_t* targ, void* workspace, size_t workspace_bytes,
+                                          int32_t rank, int64_t limit_cycles, void* stream);
+
 /* Static description of a status code. */
 const char* cure_status_string(cure_status s);
 

@@ -112,9 +112,10 @@ struct LmPlan {
   size_t ws_bytes = 0;  // per-range (max, id) partials: groups * rows * 8 bytes
 };
 LmPlan plan_lm_head(int rows, int vocab);
+// expire_rank 0 or 1 (self-test): a wait in that CTA of each pair runs out after expire_limit cycles.
 cudaError_t launch_lm_head_argmax(const LmPlan& p, const uint16_t* hidden, const uint16_t* w_lm, int rows, int d,
                                   int vocab, int32_t* out, const int32_t* out_index, void* workspace, int* err,
-                                  cudaStream_t s);
+                                  cudaStream_t s, int expire_rank = -1, long long expire_limit = 0);
 
 // Tree attention: workspace layout for a shape.
 struct AttnPlan {

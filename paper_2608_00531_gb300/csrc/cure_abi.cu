@@ -260,10 +260,9 @@ size_t cure_lm_head_workspace_size(int32_t rows, int32_t vocab) {
   return plan_lm_head(rows, vocab).ws_bytes;
 }
 
-cure_status cure_lm_head_argmax(const void* hidden, const void* w_lm, int32_t rows, int32_t d_model,
-                                int32_t vocab, const int32_t* out_index, int32_t* targ, void* workspace,
-                                size_t workspace_bytes, void* stream) {
-  ApiRange range("cure_lm_head_argmax");
+static cure_status lm_head_argmax(const void* hidden, const void* w_lm, int32_t rows, int32_t d_model, int32_t vocab,
+                                  const int32_t* out_index, int32_t* targ, void* workspace, size_t workspace_bytes,
+                                  void* stream, int expire_rank, int64_t expire_limit) {
   if (rows < 0 || d_model < 64 || vocab < 1) return CURE_ERR_INVALID_ARG;
   if (d_model % 64 != 0) return CURE_ERR_UNSUPPORTED;
   if (rows == 0) return CURE_OK;
@@ -275,7 +274,22 @@ cure_status cure_lm_head_argmax(const void* hidden, const void* w_lm, int32_t ro
   return from_cuda(launch_lm_head_argmax(plan, static_cast<const uint16_t*>(hidden),
                                          static_cast<const uint16_t*>(w_lm), rows, d_model, vocab, targ,
                                          out_index, workspace, device_error_word(),
-                                         static_cast<cudaStream_t>(stream)));
+                                         static_cast<cudaStream_t>(stream), expire_rank, expire_limit));
+}
+
+cure_status cure_lm_head_argmax(const void* hidden, const void* w_lm, int32_t rows, int32_t d_model,
+                                int32_t vocab, const int32_t* out_index, int32_t* targ, void* workspace,
+                                size_t workspace_bytes, void* stream) {
+  ApiRange range("cure_lm_head_argmax");
+  return lm_head_argmax(hidden, w_lm, rows, d_model, vocab, out_index, targ, workspace, workspace_bytes, stream, -1, 0);
+}
+
+cure_status cure_selftest_lm_head_timeout(const void* hidden, const void* w_lm, int32_t rows, int32_t d_model,
+                                          int32_t vocab, int32_t* targ, void* workspace, size_t workspace_bytes,
+                                          int32_t rank, int64_t limit_cycles, void* stream) {
+  if (rank < 0 || rank > 1 || limit_cycles < 1 || limit_cycles > (1LL << 30)) return CURE_ERR_INVALID_ARG;
+  return lm_head_argmax(hidden, w_lm, rows, d_model, vocab, nullptr, targ, workspace, workspace_bytes, stream, rank,
+                        limit_cycles);
 }
 
 cure_status cure_accept(const void* target_logits, int32_t* targ, int32_t batch, int32_t n_max,

@@ -26,7 +26,7 @@
 // writes one (max, id) per row for its vocab range; a second kernel takes the
 // first maximum over the ranges.  Waits are bounded: on expiry a CTA flags
 // CURE_DEVERR_TIMEOUT, drains its copies and products, frees its TMEM and
-// leaves.
+// leaves, and its pair reports no maximum for the range.
 //
 // What bounds it: with one tile of rows the weight's bytes (21 x 4096 x 128256:
 // 159 us, 6.6 TB/s); with several the tensor pipe at the clock that the power
@@ -64,7 +64,7 @@ constexpr int kEpiWarps = 8;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kABytes = BV * BK * 2;  // 16 KiB
 enum { B_FULL = 0, B_EMPTY = kMaxStages, B_ACCFULL = 2 * kMaxStages, B_ACCEMPTY = B_ACCFULL + 2,
-       B_DRAIN = B_ACCEMPTY + 2, kNumBars = B_DRAIN + 1 };
+       B_DRAIN = B_ACCEMPTY + 2, B_NEVER = B_DRAIN + 1, kNumBars = B_NEVER + 1 };
 constexpr int kOffBars = 0;
 constexpr int kOffTmemSlot = 8 * kNumBars;
 constexpr int kOffAbort = kOffTmemSlot + 4;
@@ -86,6 +86,8 @@ struct LmArgs {
   float* part_val;          // [groups][M] maxima
   int32_t* part_idx;        // [groups][M]
   int* err;
+  int expire_rank;          // self-test: this CTA of each pair lets an epilogue wait run out (-1: none)
+  long long expire_limit;   // after this many cycles
 };
 
 // The warp's maximum (NaNs passed over), in every lane: one instruction.
@@ -197,6 +199,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
       mbar_init(bar(B_ACCEMPTY + a), 2 * kEpiWarps);  // one arrival per epilogue warp of the pair
     }
     mbar_init(bar(B_DRAIN), 1);
+    mbar_init(bar(B_NEVER), 1);  // nothing arrives on it
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -352,6 +355,8 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
       __syncwarp();
       if (lane == 0) arrive_cluster(in_first_cta(bar(B_ACCEMPTY + a)));
     }
+    if (A.expire_rank == rank)
+      ok = __all_sync(0xffffffffu, wait_bounded(bar(B_NEVER), 0, abort_flag, A.err, true, A.expire_limit));
     // the pair's maxima meet in the first CTA's ring, which nothing writes or
     // reads any more once the last accumulator is complete: [8 quarters][256]
     // maxima, then ids
@@ -371,8 +376,12 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
   __syncwarp();
   tc_fence_before();
   __syncthreads();
+  // the pair gives up together: with a wait run out in either CTA the ring need not
+  // hold maxima, and the range reports none, so that no stale word becomes a token
+  if (threadIdx.x == 0 && *abort_flag) st_cluster(in_first_cta(sb + kOffAbort), 1u);
   cluster_sync();
-  if (rank == 0 && !*abort_flag && (int)threadIdx.x < A.nt && n0 + (int)threadIdx.x < A.M) {
+  if (rank == 0 && (int)threadIdx.x < A.nt && n0 + (int)threadIdx.x < A.M) {
+    const bool whole = !*abort_flag;
     const float* vals = reinterpret_cast<const float*>(smem + kOffRing) + threadIdx.x;
     const int* ids = reinterpret_cast<const int*>(vals) + 8 * BN;
     float best = -INFINITY;
@@ -381,7 +390,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
     for (int p = 0; p < 8; ++p) {
       const float v = vals[p * BN];
       const int i = ids[p * BN];
-      if (i >= 0 && (v > best || (v == best && i < b))) {
+      if (whole && i >= 0 && (v > best || (v == best && i < b))) {
         best = v;
         b = i;
       }
@@ -479,7 +488,7 @@ LmPlan plan_lm_head(int rows, int vocab) {
 
 cudaError_t launch_lm_head_argmax(const LmPlan& p, const uint16_t* hidden, const uint16_t* w_lm, int rows, int d,
                                   int vocab, int32_t* out, const int32_t* out_index, void* workspace, int* err,
-                                  cudaStream_t s) {
+                                  cudaStream_t s, int expire_rank, long long expire_limit) {
   if (rows == 0) return cudaSuccess;
   static std::atomic<uint64_t> attr_done{0};
   int dev = 0;
@@ -506,6 +515,8 @@ cudaError_t launch_lm_head_argmax(const LmPlan& p, const uint16_t* hidden, const
   a.part_val = static_cast<float*>(workspace);
   a.part_idx = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + (size_t)p.groups * rows * sizeof(float));
   a.err = err;
+  a.expire_rank = expire_rank;
+  a.expire_limit = expire_limit;
   e = launch_pdl(lm_head_argmax_kernel, dim3(2 * p.n_tiles * p.groups), dim3(kThreads),
                  1024 + kOffRing + a.stages * stage_bytes(p.nt), s, mh, mw, a);
   if (e != cudaSuccess) return e;

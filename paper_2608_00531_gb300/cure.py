@@ -317,6 +317,17 @@ def cure_selftest_wait_timeout(limit_cycles: int = 1 << 24, stream=None) -> None
     check("cure_selftest_wait_timeout", _lib.load().cure_selftest_wait_timeout(int(limit_cycles), _stream(stream)))
 
 
+def cure_selftest_lm_head_timeout(hidden: torch.Tensor, w_lm: torch.Tensor, rank: int, out: torch.Tensor,
+                                  workspace: torch.Tensor, limit_cycles: int = 1 << 22, *, stream=None) -> torch.Tensor:
+    """cure_lm_head_argmax with a wait that runs out in one CTA of every pair (a
+    failure-detection self-test); read the outcome with cure_device_error()."""
+    rows, d = hidden.shape
+    check("cure_selftest_lm_head_timeout", _lib.load().cure_selftest_lm_head_timeout(
+        _p(hidden), _p(w_lm), rows, d, w_lm.shape[0], _p(out), _p(workspace),
+        workspace.numel() * workspace.element_size(), int(rank), int(limit_cycles), _stream(stream)))
+    return out
+
+
 def cure_status_string(code: int) -> str:
     return _lib.load().cure_status_string(code).decode()
 

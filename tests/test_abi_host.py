@@ -216,3 +216,6 @@ def test_selftest_limit_is_checked_on_the_host(lib):
     others are refused before any launch."""
     for bad in (0, -5, (1 << 30) + 1):
         assert lib.cure_selftest_wait_timeout(bad, None) == 1
+        assert lib.cure_selftest_lm_head_timeout(None, None, 1, 64, 10, None, None, 256, 0, bad, None) == 1
+    for rank in (-1, 2):
+        assert lib.cure_selftest_lm_head_timeout(None, None, 1, 64, 10, None, None, 256, rank, 100, None) == 1

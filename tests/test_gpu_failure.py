@@ -42,3 +42,26 @@ def test_bounded_wait_reports_a_timeout_and_the_context_stays_usable(cure):
     assert np.array_equal(ids.cpu().numpy(), o_ids)
     assert np.array_equal(margin.cpu().numpy(), o_m.astype(np.float32))
     assert cure.cure_device_error() == 0
+
+
+@pytest.mark.parametrize("rank", [0, 1])
+@pytest.mark.parametrize("rows,d,V", [(21, 128, 5000), (300, 64, 40000)])
+def test_lm_head_timeout_in_either_cta_of_a_pair_leaves_ids_of_the_vocabulary(cure, rank, rows, d, V):
+    """A wait that runs out in one CTA of a pair after the products are done: the
+    pair has no maxima to report.  Neither ring contents nor what the workspace
+    held (here large values with an impossible id) may become a token; the next
+    call on the same workspace is right again."""
+    from paper_2608_00531_gb300 import _lib
+    rng = np.random.default_rng(rows + rank)
+    # hidden states far below the weights: every logit is smaller than the words in the ring
+    h = W.to_bf16((rng.standard_normal((rows, d)) * 1e-3).astype(np.float32)).to(DEV)
+    w = W.to_bf16((rng.standard_normal((V, d)) / np.sqrt(d)).astype(np.float32)).to(DEV)
+    ws = torch.full((cure.cure_lm_head_workspace_size(rows, V) // 4,), 0x7f000000, dtype=torch.int32, device=DEV)
+    out = torch.full((rows,), -7, dtype=torch.int32, device=DEV)
+    assert cure.cure_device_error() == 0
+    cure.cure_selftest_lm_head_timeout(h, w, rank, out, ws)
+    assert cure.cure_device_error() == _lib.DEVERR_TIMEOUT
+    assert ((out >= 0) & (out < V)).all()
+    good = cure.cure_lm_head_argmax(h, w, workspace=ws)
+    assert cure.cure_device_error() == 0
+    assert torch.equal(good, cure.cure_lm_head_argmax(h, w))
