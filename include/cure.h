@@ -348,6 +348,16 @@ cure_status cure_selftest_lm_head_timeout(const void* hidden, const void* w_lm, 
                                           int32_t vocab, int32_t* targ, void* workspace, size_t workspace_bytes,
                                           int32_t rank, int64_t limit_cycles, void* stream);
 
+/*
+ * Self-test: the form a cure_tree_attn call of this shape takes (`kv` and
+ * `route` are HOST pointers; in_place != 0: the in-place layout).  route[0] is
+ * the number of CTAs in each unit's cluster (0: the persistent form), route[1]
+ * is 1 if that takes its pieces in two tile slots in turn, route[2] the CTAs
+ * of the grid.
+ */
+cure_status cure_selftest_attn_route(int32_t batch, int32_t n_max, int32_t heads_q, const cure_kv_desc* kv,
+                                     int32_t in_place, int32_t* route);
+
 /* Static description of a status code. */
 const char* cure_status_string(cure_status s);
 

@@ -20,7 +20,8 @@ DEVERR_PAGE, DEVERR_SLOT, DEVERR_NODES, DEVERR_TOKEN, DEVERR_TIMEOUT = 0x1, 0x2,
 # every entry point the header declares
 EXPORTS = ("cure_score_draft", "cure_build_tree", "cure_tree_attn", "cure_tree_attn_workspace_size",
            "cure_accept", "cure_lm_head_argmax", "cure_lm_head_workspace_size", "cure_selftest_wait_timeout",
-           "cure_selftest_lm_head_timeout", "cure_sample_target", "cure_resync_kv", "cure_device_error",
+           "cure_selftest_lm_head_timeout", "cure_selftest_attn_route",
+           "cure_sample_target", "cure_resync_kv", "cure_device_error",
            "cure_status_string", "cure_abi_version")
 
 
@@ -74,6 +75,8 @@ def load() -> C.CDLL:
     lib.cure_selftest_wait_timeout.restype = C.c_int
     lib.cure_selftest_lm_head_timeout.argtypes = [P, P, I32, I32, I32, P, P, C.c_size_t, I32, C.c_int64, P]
     lib.cure_selftest_lm_head_timeout.restype = C.c_int
+    lib.cure_selftest_attn_route.argtypes = [I32, I32, I32, C.POINTER(KVDesc), I32, C.POINTER(I32)]
+    lib.cure_selftest_attn_route.restype = C.c_int
     lib.cure_resync_kv.argtypes = [I32, C.POINTER(C.c_void_p), C.POINTER(C.c_void_p),
                                    C.POINTER(KVDesc), P, P, I32, I32, I32, P, P, P, P, P, P, P,
                                    P, P, P]

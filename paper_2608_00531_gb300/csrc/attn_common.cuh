@@ -53,7 +53,18 @@ constexpr int kAttnMaxCluster = 16;
 // form for `units` units of up to `tiles` tiles, else 0 (stream-K).
 int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged);
 
-// The persistent tcgen05 kernel (writes `out`; merges split units itself).
-cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s);
+// Whether the persistent form of `ctas` CTAs takes its pieces in the two M tile
+// slots in turn (one_tile: every unit fits one M tile).
+bool attn_ping_pong(int units, int ctas, bool one_tile);
+
+// The form a call takes.
+struct AttnRoute {
+  int cluster;     // CTAs of each unit's cluster; 0: the persistent form
+  bool ping_pong;  // persistent, the two M tile slots in turn
+  int ctas;        // of the grid
+};
+
+// The tcgen05 kernel in that form (writes `out`; merges split units itself).
+cudaError_t launch_tree_attn_tc(const AttnArgs& A, const AttnRoute& route, cudaStream_t s);
 
 }  // namespace cure

@@ -32,6 +32,36 @@ bool plan_tree_attn(int batch, int n_max, int heads_q, const cure_kv_desc& kv, A
   return true;
 }
 
+namespace {
+
+// The rules on shapes alone that pick a call's form: a cluster per unit, or the
+// persistent grid.
+AttnRoute route_of(const AttnPlan& plan, const cure_kv_desc& kv, int batch, int n_max, int heads_q, bool inplace) {
+  const int G = heads_q / kv.heads_kv;
+  const int cap = kv.layout == 0 ? kv.max_len : kv.max_len * kv.page_size;
+  const int64_t tiles_unit = (cap + kAttnKeys - 1) / kAttnKeys +
+                             (inplace ? 0 : (n_max + kAttnKeys - 1) / kAttnKeys);
+  const int64_t positions = (int64_t)plan.units_max * (tiles_unit + kAttnUnitCost);
+  AttnRoute r{};
+  r.cluster = attn_cluster_size(plan.units_max, tiles_unit, n_max > kAttnRowsCta / G, batch > 1);
+  if (r.cluster > 0) {
+    r.ctas = plan.units_max * r.cluster;
+    return r;
+  }
+  // One CTA per SM, unless the shape's work (bounded above from the cache
+  // capacity, since the lengths are on the device) gives a CTA fewer than
+  // kAttnMinTiles tile positions: a unit cut into many pieces costs a merge of
+  // that many partials, which the last piece does alone, so small problems
+  // take fewer, longer pieces.
+  r.ctas = std::min(num_sms(), kAttnMaxCtas);
+  if (kAttnMinTiles > 0)
+    r.ctas = (int)std::max<int64_t>(1, std::min<int64_t>(r.ctas, positions / kAttnMinTiles));
+  r.ping_pong = attn_ping_pong(plan.units_max, r.ctas, n_max <= kAttnRowsCta / G);
+  return r;
+}
+
+}  // namespace
+
 cudaError_t launch_tree_attn(const AttnPlan& plan, const uint16_t* q, const uint16_t* tree_k,
                              const uint16_t* tree_v, const uint16_t* k_cache,
                              const uint16_t* v_cache, const cure_kv_desc& kv,
@@ -65,20 +95,24 @@ cudaError_t launch_tree_attn(const AttnPlan& plan, const uint16_t* q, const uint
   A.ws_lse = reinterpret_cast<float*>(ws + plan.ws_cnt + plan.ws_o);
   A.out = out;
   A.err = err;
-  // One CTA per SM, unless the shape's work (bounded above from the cache
-  // capacity, since the lengths are on the device) gives a CTA fewer than
-  // kAttnMinTiles tile positions: a unit cut into many pieces costs a merge of
-  // that many partials, which the last piece does alone, so small problems
-  // take fewer, longer pieces.
-  const int64_t tiles_unit = (A.cap + kAttnKeys - 1) / kAttnKeys +
-                             (A.inplace ? 0 : (n_max + kAttnKeys - 1) / kAttnKeys);
-  const int64_t positions = (int64_t)plan.units_max * (tiles_unit + kAttnUnitCost);
-  A.cluster = attn_cluster_size(plan.units_max, tiles_unit, n_max > kAttnRowsCta / A.G, batch > 1);
-  if (A.cluster > 0) return launch_tree_attn_tc(A, dim3(plan.units_max * A.cluster, 1, 1), s);
-  int ctas = std::min(num_sms(), kAttnMaxCtas);
-  if (kAttnMinTiles > 0)
-    ctas = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, positions / kAttnMinTiles));
-  return launch_tree_attn_tc(A, dim3(ctas, 1, 1), s);
+  const AttnRoute r = route_of(plan, kv, batch, n_max, heads_q, A.inplace);
+  A.cluster = r.cluster;
+  return launch_tree_attn_tc(A, r, s);
 }
 
 }  // namespace cure
+
+using namespace cure;
+
+extern "C" cure_status cure_selftest_attn_route(int32_t batch, int32_t n_max, int32_t heads_q, const cure_kv_desc* kv,
+                                                int32_t in_place, int32_t* route) {
+  AttnPlan plan;
+  if (!route || batch < 1 || cure_tree_attn_workspace_size(batch, n_max, heads_q, kv) == 0 ||
+      !plan_tree_attn(batch, n_max, heads_q, *kv, &plan))
+    return CURE_ERR_INVALID_ARG;
+  const AttnRoute r = route_of(plan, *kv, batch, n_max, heads_q, in_place != 0);
+  route[0] = r.cluster;
+  route[1] = r.ping_pong;
+  route[2] = r.ctas;
+  return CURE_OK;
+}

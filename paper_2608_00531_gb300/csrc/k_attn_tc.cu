@@ -1435,7 +1435,19 @@ int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
   return size;
 }
 
-cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
+// Ping-pong where every unit fits one M tile and a CTA has at least 1.5 units
+// on average: it hides the pieces' starts and ends.  us per call, stream-K ->
+// ping-pong (sequences x kv heads of query heads, keys; units a CTA):
+//   64 x 8 of 4, 200-300 (3.4)        47.0 -> 41.0
+//   16 x 16 of 1, 500-900 (1.7)       36.6 -> 34.2
+//   60 x 16 of 1, 1000-2000 (6.3)    144.5 -> 143.0
+//   32 x 8 of 4, 1024-8192 (1.7)     113.3 -> 108.2
+//   15 x 16 of 1, 32768 (1.6)          651 -> 631
+// With fewer pieces there is little to hide: 16 x 8 of 4, 1024-8192 (0.84) 62.2 ->
+// 62.4; 20 x 8 of 5, 3000-9000 (1.05) 87.7 -> 87.9.
+bool attn_ping_pong(int units, int ctas, bool one_tile) { return one_tile && 2 * (int64_t)units >= 3 * (int64_t)ctas; }
+
+cudaError_t launch_tree_attn_tc(const AttnArgs& A, const AttnRoute& route, cudaStream_t s) {
   cudaError_t e = set_attributes();
   if (e != cudaSuccess) return e;
   const int Hkv = A.kv.heads_kv;
@@ -1463,23 +1475,12 @@ cudaError_t launch_tree_attn_tc(const AttnArgs& A, dim3 grid, cudaStream_t s) {
   AttnArgs a = A;
   a.tag = launches.fetch_add(1) % ((1u << (32 - kCountBits)) - 1) + 1;
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg = cluster_config(attr, grid, A.cluster > 0 ? A.cluster : 1);
+  cudaLaunchConfig_t cfg = cluster_config(attr, dim3(route.ctas), A.cluster > 0 ? A.cluster : 1);
   cfg.stream = s;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see pdl_begin()
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;
-  // Ping-pong where every unit fits one M tile and a CTA has at least 1.5 units
-  // on average: it hides the pieces' starts and ends.  us per call, stream-K ->
-  // ping-pong (sequences x kv heads of query heads, keys; units a CTA):
-  //   64 x 8 of 4, 200-300 (3.4)        47.0 -> 41.0
-  //   16 x 16 of 1, 500-900 (1.7)       36.6 -> 34.2
-  //   60 x 16 of 1, 1000-2000 (6.3)    144.5 -> 143.0
-  //   32 x 8 of 4, 1024-8192 (1.7)     113.3 -> 108.2
-  //   15 x 16 of 1, 32768 (1.6)          651 -> 631
-  // With fewer pieces there is little to hide: 16 x 8 of 4, 1024-8192 (0.84) 62.2 ->
-  // 62.4; 20 x 8 of 5, 3000-9000 (1.05) 87.7 -> 87.9.
-  const bool one_tile = A.n_max <= BM / A.G;
-  const int mode = A.cluster > 0 ? kCluster : one_tile && 2 * (int64_t)A.units_max >= 3 * (int64_t)grid.x ? kPingPong : kStreamK;
+  const int mode = A.cluster > 0 ? kCluster : route.ping_pong ? kPingPong : kStreamK;
   e = cudaLaunchKernelEx(&cfg, kKernels[mode][A.inplace ? 1 : 0], mk, mv, mtk, mtv, mq, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

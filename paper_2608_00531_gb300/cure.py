@@ -328,6 +328,15 @@ def cure_selftest_lm_head_timeout(hidden: torch.Tensor, w_lm: torch.Tensor, rank
     return out
 
 
+def cure_selftest_attn_route(batch: int, n_max: int, heads_q: int, kv: KVDesc, in_place: bool) -> tuple[int, bool, int]:
+    """The form a tree-attention call of this shape takes: CTAs per unit's cluster
+    (0: persistent), pieces in two tile slots in turn, CTAs of the grid."""
+    r = (C.c_int32 * 3)()
+    check("cure_selftest_attn_route",
+          _lib.load().cure_selftest_attn_route(batch, n_max, heads_q, C.byref(kv), int(in_place), r))
+    return r[0], bool(r[1]), r[2]
+
+
 def cure_status_string(code: int) -> str:
     return _lib.load().cure_status_string(code).decode()
 

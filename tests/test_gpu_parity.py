@@ -385,6 +385,13 @@ def _run_attn(c, t, q, tk, tv, kc, vc, L, table, npages, Hkv):
     return out.float().cpu().numpy()
 
 
+def _route(c, q, kc, table, npages, Hkv, in_place):
+    """The form the call takes: CTAs per unit's cluster (0: persistent), ping-pong, grid."""
+    kv = c.kv_desc(Hkv, 128, kc.shape[1]) if table is None else \
+        c.kv_desc(Hkv, 128, table.shape[1], torch.from_numpy(table).to(DEV), kc.shape[1], npages)
+    return c.cure_selftest_attn_route(q.shape[0], q.shape[1], q.shape[2], kv, in_place)
+
+
 def _cmp_attn(got, ref, t, seqs=None):
     B = got.shape[0]
     worst = 0.0
@@ -429,17 +436,23 @@ def test_tree_attn_page_sizes(cure, ps, Hq, Hkv):
 
 @pytest.mark.parametrize("in_place", [False, True])
 @pytest.mark.parametrize("paged", [False, True])
-@pytest.mark.parametrize("B,Hq,Hkv,lens", [
-    (1, 4, 1, (3,)),                       # one unit, fewer tiles than the 16 CTAs of its cluster
-    (2, 8, 2, (0, 1100)),                  # 16 CTAs a unit, one sequence with an empty cache
-    (1, 32, 8, (700,)),                    # 8
-    (4, 32, 8, (64, 1, 129, 600)),         # 4, ragged
-    (9, 32, 8, (300, 20, 64, 0, 5, 63, 65, 128, 250)),  # 2 (72 units)
-    (1, 64, 1, (500,)),                    # one sequence in several row groups
+@pytest.mark.parametrize("B,Hq,Hkv,lens,lo,hi", [
+    (1, 4, 1, (3,), 3, 4),                 # one unit, fewer tiles than its cluster has CTAs
+    (2, 8, 2, (0, 1100), 9, 12),           # one sequence with an empty cache: one tile, the other CTAs none
+    (1, 32, 8, (700,), 9, 12),
+    (4, 32, 8, (64, 1, 129, 600), 4, 4),   # ragged
+    (9, 32, 8, (300, 20, 64, 0, 5, 63, 65, 128, 250), 2, 2),  # 72 units
+    (1, 64, 1, (500,), 9, 12),             # one sequence in several row groups of two M tiles
+    (2, 32, 8, (500, 60), 5, 8),           # one M tile
+    (1, 56, 8, (300,), 5, 8),              # two
+    (1, 16, 4, (3000,), 13, 16),
+    (2, 8, 2, (20, 2000), 13, 16),         # one sequence with far fewer tiles than CTAs
 ])
-def test_tree_attn_few_units(cure, B, Hq, Hkv, lens, paged, in_place):
-    """Problems small enough for a cluster of CTAs per unit: every cluster
-    size, CTAs without a tile, empty caches, one and two M tiles, row groups."""
+def test_tree_attn_few_units(cure, B, Hq, Hkv, lens, lo, hi, paged, in_place):
+    """Problems small enough for a cluster of CTAs per unit.  lo and hi bound the
+    CTAs a unit gets: sizes on both sides of 4 and 8, up to which the merge is
+    compiled apart, the smallest and the largest; CTAs without a tile, empty
+    caches, one and two M tiles, row groups."""
     if in_place:
         t, q, kc, vc, L, table, npages = _in_place_case(B, 16, 8, Hq, Hkv, list(lens), paged, seed=B + Hq)
         tk = tv = None
@@ -448,6 +461,7 @@ def test_tree_attn_few_units(cure, B, Hq, Hkv, lens, paged, in_place):
         t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 16, 8, Hq, Hkv, list(lens), paged, 1.0, 1.0, seed=B + Hq)
         got = _run_attn(cure, t, q, tk, tv, kc, vc, L, table, npages, Hkv)
         tk, tv = _f64(tk), _f64(tv)
+    assert lo <= _route(cure, q, kc, table, npages, Hkv, in_place)[0] <= hi
     ref = oracle.tree_attn(_f64(q), tk, tv, _f64(kc), _f64(vc), L, t["n_nodes"], t["anc"], 1.0 / math.sqrt(128),
                            table, 16)
     _cmp_attn(got, ref, t)
@@ -497,7 +511,7 @@ def test_tree_attn_many_one_tile_units(cure, Hq, Hkv, paged, in_place):
         tk = tv = None
     else:
         t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 12, 8, Hq, Hkv, lens, paged, 1.0, 1.0, seed=Hq)
-    assert q.shape[1] <= 128 // (Hq // Hkv)
+    assert _route(cure, q, kc, table, npages, Hkv, in_place)[:2] == (0, True)
     kv = cure.kv_desc(Hkv, 128, table.shape[1], torch.from_numpy(table).to(DEV), 16, npages) if paged else \
         cure.kv_desc(Hkv, 128, kc.shape[1])
     ws = torch.randint(0, 256, (cure.cure_tree_attn_workspace_size(B, q.shape[1], Hq, kv),), dtype=torch.uint8,
@@ -528,6 +542,7 @@ def test_tree_attn_short_pieces_before_long_ones(cure, paged, in_place):
         tk = tv = None
     else:
         t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 12, 8, Hq, Hkv, lens, paged, 1.0, 1.0, seed=11)
+    assert _route(cure, q, kc, table, npages, Hkv, in_place)[:2] == (0, True)
     ref = oracle.tree_attn(_f64(q), None if tk is None else _f64(tk), None if tv is None else _f64(tv), _f64(kc),
                            _f64(vc), L, t["n_nodes"], t["anc"], 1.0 / math.sqrt(128), table, 16)
     for _ in range(3):
@@ -544,6 +559,7 @@ def test_tree_attn_split_units_on_garbage_workspace(cure, paged):
     ranges merge through the workspace, whatever it holds on entry."""
     lens = [900, 37, 1500, 64, 300, 0, 1100, 700, 129, 2000, 511, 1024]
     t, q, tk, tv, kc, vc, L, table, npages = _attn_case(12, 16, 8, 32, 8, lens, paged, 1.0, 1.0, seed=9)
+    assert _route(cure, q, kc, table, npages, 8, False)[:2] == (0, False)
     kv = cure.kv_desc(8, 128, table.shape[1], torch.from_numpy(table).to(DEV), 16, npages) if paged else \
         cure.kv_desc(8, 128, kc.shape[1])
     ref = oracle.tree_attn(_f64(q), _f64(tk), _f64(tv), _f64(kc), _f64(vc), L, t["n_nodes"], t["anc"],
@@ -663,6 +679,8 @@ def test_tree_attn_rows_that_see_no_key(cure, B, Hkv, n, in_place):
         anc[:, :n, a >> 6] |= bits[:, :, a].astype(np.uint64) << np.uint64(a & 63)
     t = dict(n_nodes=np.full(B, n, dtype=np.int32), anc=anc)
     L = np.zeros(B, dtype=np.int32)
+    cluster, ping_pong, _ = _route(cure, q, kc, None, 0, Hkv, in_place)
+    assert (cluster > 0, ping_pong) == (B == 2, B == 30)
     got = _run_attn_in_place(cure, t, q, kc, vc, L, None, 0, Hkv) if in_place else \
         _run_attn(cure, t, q, tk, tv, kc, vc, L, None, 0, Hkv)
     k, v = _f64(tk)[:, :n], _f64(tv)[:, :n]
