@@ -104,7 +104,7 @@ def test_lm_head_argmax_tile_edges(cure, rows, d, V):
 
 
 def test_lm_head_argmax_more_m_tiles_than_sms(cure):
-    """More 128-row tiles than SMs: one vocab range per tile and a grid of
+    """More 256-row tiles than SM pairs: one vocab range per tile and a grid of
     more than one wave."""
     rng = np.random.default_rng(8)
     rows, d, V = 160 * 128 + 37, 64, 700
@@ -115,6 +115,35 @@ def test_lm_head_argmax_more_m_tiles_than_sms(cure):
     sel = np.concatenate([np.arange(64), rows - 64 + np.arange(64), rng.choice(rows, 128, replace=False)])
     exact = _check(got[sel], W.bf16_to_f64(h)[sel], W.bf16_to_f64(w), d)
     assert exact >= 0.8 * len(sel)
+
+
+@pytest.mark.parametrize("rows,d,V", [(21, 128, 5000), (300, 64, 1000)])
+def test_lm_head_argmax_nan_and_infinite_logits(cure, rows, d, V):
+    """A NaN logit is passed over, +inf is a maximum like another (the lowest id
+    wins), and a row without a logit above -inf gives id 0."""
+    rng = np.random.default_rng(rows)
+    h = rng.standard_normal((rows, d)).astype(np.float32)
+    w = (rng.standard_normal((V, d)) / np.sqrt(d)).astype(np.float32)
+    h[:, :3] = 0.0
+    w[:, :3] = 0.0
+    h[0::5, 0] = 1.0                      # these rows' logits at ids 40, 700 are +inf
+    w[40, 0] = w[700, 0] = np.inf         # (0 * inf: NaN for every other row)
+    h[1::5] = np.nan                      # nothing but NaNs
+    h[2::5, 1] = 3.0
+    w[V - 1, 1] = -np.inf                 # -inf there, NaN elsewhere
+    hb, wb = W.to_bf16(h), W.to_bf16(w)
+    got = cure.cure_lm_head_argmax(hb.to(DEV), wb.to(DEV)).cpu().numpy()
+    assert cure.cure_device_error() == 0
+    with np.errstate(invalid="ignore"):
+        lg = np.einsum("rd,vd->rv", W.bf16_to_f64(hb), W.bf16_to_f64(wb))
+    assert (got[0::5] == 40).all() and (got[1::5] == 0).all()
+    for r in [r for r in range(rows) if r % 5 > 1]:
+        row = lg[r]
+        assert not np.isnan(row[got[r]]) and row[got[r]] >= np.nanmax(row) - 2e-4, r  # twice the bound above at sum |h w| < 16
+    h2 = np.abs(h[2:3]).repeat(2, 0)      # every logit -inf
+    w2 = np.full((V, d), -np.inf, dtype=np.float32)
+    got = cure.cure_lm_head_argmax(W.to_bf16(h2 + 1).to(DEV), W.to_bf16(w2).to(DEV)).cpu().numpy()
+    assert (got == 0).all()
 
 
 def test_lm_head_argmax_ties_take_the_lowest_id(cure):
