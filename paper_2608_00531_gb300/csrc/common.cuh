@@ -42,6 +42,11 @@ __device__ __forceinline__ void flag(int* err, int bits) {
 // kernel's tail); every kernel calls pdl_begin() before its first read of
 // global memory, which waits for the previous kernel to complete and lets
 // the next one be scheduled.  Without a programmatic launch both are no-ops.
+// The wait comes before the trigger: once a kernel runs, everything before the
+// kernel that it follows has completed.  The acceptance walk behind the target
+// argmax of the same call relies on that (it reads the tree before its own
+// pdl_begin()), so that argmax must neither trigger earlier nor write anything
+// that the walk reads but targ.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -361,9 +361,9 @@ cudaError_t launch_accept_walk(int batch, int n_max, int block, const int32_t* n
                                int32_t* diverge_depth, bool after_argmax, int* err, cudaStream_t s) {
   if (batch == 0) return cudaSuccess;
   const int grid = (batch + kWarpsPerCta - 1) / kWarpsPerCta;
-  return launch_pdl(after_argmax ? accept_walk_kernel<true> : accept_walk_kernel<false>, dim3(grid), dim3(32 * kWarpsPerCta), 0, s, batch, n_max, block,
-                    n_nodes, tok, parent, depth, anc, targ, accept_len, best_node, path_nodes,
-                    out_tokens, diverge_depth, err);
+  return launch_pdl(after_argmax ? accept_walk_kernel<true> : accept_walk_kernel<false>, dim3(grid),
+                    dim3(32 * kWarpsPerCta), 0, s, batch, n_max, block, n_nodes, tok, parent, depth, anc, targ,
+                    accept_len, best_node, path_nodes, out_tokens, diverge_depth, err);
 }
 
 }  // namespace cure

@@ -259,7 +259,7 @@ __device__ __forceinline__ void cluster_wait() {
 __global__ void __launch_bounds__(kCtaThreads, 6)
 vocab_ring_kernel(const uint16_t* __restrict__ logits, int vocab, int n_max, const int32_t* __restrict__ n_nodes,
                   int32_t* __restrict__ targ, int* err) {
-  pdl_begin();
+  pdl_begin();  // (accept_walk_kernel counts on the wait in here coming before the trigger)
   const int64_t row = blockIdx.y;
   const int S = gridDim.x;
   const int c = blockIdx.x;  // rank within the cluster
