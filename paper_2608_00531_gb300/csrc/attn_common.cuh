@@ -54,8 +54,9 @@ constexpr int kAttnMaxCluster = 16;
 int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged);
 
 // Whether the persistent form of `ctas` CTAs takes its pieces in the two M tile
-// slots in turn (one_tile: every unit fits one M tile).
-bool attn_ping_pong(int units, int ctas, bool one_tile);
+// slots in turn (one_tile: every unit fits one M tile; small_pages: a cache in
+// pages of up to 16 tokens).
+bool attn_ping_pong(int units, int ctas, bool one_tile, bool small_pages);
 
 // The form a call takes.
 struct AttnRoute {

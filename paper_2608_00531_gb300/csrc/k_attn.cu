@@ -56,7 +56,8 @@ AttnRoute route_of(const AttnPlan& plan, const cure_kv_desc& kv, int batch, int 
   r.ctas = std::min(num_sms(), kAttnMaxCtas);
   if (kAttnMinTiles > 0)
     r.ctas = (int)std::max<int64_t>(1, std::min<int64_t>(r.ctas, positions / kAttnMinTiles));
-  r.ping_pong = attn_ping_pong(plan.units_max, r.ctas, n_max <= kAttnRowsCta / G);
+  r.ping_pong = attn_ping_pong(plan.units_max, r.ctas, n_max <= kAttnRowsCta / G,
+                               kv.layout == 1 && kv.page_size <= 16);
   return r;
 }
 

@@ -1435,17 +1435,24 @@ int attn_cluster_size(int units, int64_t tiles, bool two_m_tiles, bool ragged) {
   return size;
 }
 
-// Ping-pong where every unit fits one M tile and a CTA has at least 1.5 units
-// on average: it hides the pieces' starts and ends.  us per call, stream-K ->
-// ping-pong (sequences x kv heads of query heads, keys; units a CTA):
-//   64 x 8 of 4, 200-300 (3.4)        47.0 -> 41.0
-//   16 x 16 of 1, 500-900 (1.7)       36.6 -> 34.2
-//   60 x 16 of 1, 1000-2000 (6.3)    144.5 -> 143.0
-//   32 x 8 of 4, 1024-8192 (1.7)     113.3 -> 108.2
-//   15 x 16 of 1, 32768 (1.6)          651 -> 631
-// With fewer pieces there is little to hide: 16 x 8 of 4, 1024-8192 (0.84) 62.2 ->
-// 62.4; 20 x 8 of 5, 3000-9000 (1.05) 87.7 -> 87.9.
-bool attn_ping_pong(int units, int ctas, bool one_tile) { return one_tile && 2 * (int64_t)units >= 3 * (int64_t)ctas; }
+// Ping-pong where every unit fits one M tile and the cache has pages of 8 or 16
+// tokens, or a CTA has at least 9/8 units on average: it hides the pieces' starts
+// and ends, and with small pages (4 to 8 copies a tile and operand) it is the
+// faster form at any number of units.  us per call, stream-K -> ping-pong
+// (sequences x kv heads of query heads, keys, page; units a CTA):
+//   64 x 8 of 4, 200-300 (3.4)            47.0 -> 41.0
+//   60 x 16 of 1, 1000-2000 (6.3)        144.5 -> 143.0
+//   32 x 8 of 4, 1024-8192, 16 (1.7)     113.3 -> 108.2
+//   28 x 8 of 4, 16000-16384 (1.5)       284.8 -> 283.0
+//   22 x 8 of 4, 1000-4000 (1.16)         44.9 -> 44.2
+//   20 x 8 of 4, 3000-9000 (1.05)         83.9 -> 84.5;  page 64 86.5 -> 86.8;  16 90.1 -> 88.0
+//   14 x 8 of 4, 7000-8192, page 32 (.74) 82.5 -> 83.2;   8 107.0 -> 104.3
+//   10 x 8 of 4, 1024-8192, page 32 (.53) 43.7 -> 44.5;  16 47.2 -> 45.9;  8 53.6 -> 52.9
+//   8 x 8 of 4, 16000-32000, 16 (.42)    139.8 -> 137.5
+//   1 x 8 of 4, 262144, 16 (.05)         206.4 -> 204.7;  contiguous 178.5 -> 181.6
+bool attn_ping_pong(int units, int ctas, bool one_tile, bool small_pages) {
+  return one_tile && (small_pages || 8 * (int64_t)units >= 9 * (int64_t)ctas);
+}
 
 cudaError_t launch_tree_attn_tc(const AttnArgs& A, const AttnRoute& route, cudaStream_t s) {
   cudaError_t e = set_attributes();

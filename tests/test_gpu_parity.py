@@ -553,13 +553,38 @@ def test_tree_attn_short_pieces_before_long_ones(cure, paged, in_place):
         _cmp_attn(got, ref, t)
 
 
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("ps,ping_pong", [(8, True), (16, True), (32, False)])
+@pytest.mark.parametrize("B,Hkv,room", [(12, 8, 0), (1, 8, 131072), (2, 4, 200000)])
+def test_tree_attn_few_one_tile_units_by_page_size(cure, B, Hkv, room, ps, ping_pong, in_place):
+    """Fewer one-tile units than SMs on the persistent form, which takes them in
+    the two tile slots in turn with pages of up to 16 tokens.  12 x 8 units are
+    too many for a cluster each; a block table with room for long sequences
+    keeps few units off clusters too, and their short sequences are cut into up
+    to 19 pieces."""
+    lens = [900, 37, 1500, 64, 300, 0, 1100, 700, 129, 2000, 511, 1024] if B == 12 else [3000, 63][:B]
+    if in_place:
+        t, q, kc, vc, L, table, npages = _in_place_case(B, 16, 8, 4 * Hkv, Hkv, lens, True, seed=ps + B, ps=ps)
+        tk = tv = None
+    else:
+        t, q, tk, tv, kc, vc, L, table, npages = _attn_case(B, 16, 8, 4 * Hkv, Hkv, lens, True, 1.0, 1.0, seed=ps + B, ps=ps)
+    table = np.pad(table, ((0, 0), (0, max(0, room // ps - table.shape[1]))), constant_values=-1)
+    assert _route(cure, q, kc, table, npages, Hkv, in_place)[:2] == (0, ping_pong)
+    ref = oracle.tree_attn(_f64(q), None if tk is None else _f64(tk), None if tv is None else _f64(tv), _f64(kc),
+                           _f64(vc), L, t["n_nodes"], t["anc"], 1.0 / math.sqrt(128), table, ps)
+    for _ in range(2):
+        got = _run_attn_in_place(cure, t, q, kc, vc, L, table, npages, Hkv) if in_place else \
+            _run_attn(cure, t, q, tk, tv, kc, vc, L, table, npages, Hkv)
+        _cmp_attn(got, ref, t)
+
+
 @pytest.mark.parametrize("paged", [False, True])
 def test_tree_attn_split_units_on_garbage_workspace(cure, paged):
     """96 units, too many for a cluster each: the units cut by the stream-K
     ranges merge through the workspace, whatever it holds on entry."""
     lens = [900, 37, 1500, 64, 300, 0, 1100, 700, 129, 2000, 511, 1024]
     t, q, tk, tv, kc, vc, L, table, npages = _attn_case(12, 16, 8, 32, 8, lens, paged, 1.0, 1.0, seed=9)
-    assert _route(cure, q, kc, table, npages, 8, False)[:2] == (0, False)
+    assert _route(cure, q, kc, table, npages, 8, False)[:2] == (0, paged)  # (16-token pages: two tile slots in turn)
     kv = cure.kv_desc(8, 128, table.shape[1], torch.from_numpy(table).to(DEV), 16, npages) if paged else \
         cure.kv_desc(8, 128, kc.shape[1])
     ref = oracle.tree_attn(_f64(q), _f64(tk), _f64(tv), _f64(kc), _f64(vc), L, t["n_nodes"], t["anc"],
