@@ -1305,3 +1305,41 @@ def test_full_step_serve_shape(cure):
             assert float((r2["attn"][:, b, :nb].float() - attn[:, b, :nb]).abs().max()) <= 1e-2, b
     row_bytes = w.vocab * 2
     assert h2d[1] - h2d[0] == int((N - t["n_nodes"]).sum()) * row_bytes
+
+
+@pytest.mark.parametrize("layer_map", [None, [0, 1, 0]])
+def test_step_attention_route_does_not_matter(cure, layer_map):
+    """A step whose layers lie in one tensor addresses them without views; with
+    q as a list, or in a larger tensor with gaps between the layers, it takes
+    them one by one: the same results, layer by layer equal to the call itself."""
+    from paper_2608_00531_gb300.step import RepairVerifyStep, StepInputs
+    B, K, R, V, layers, Hq, Hkv = 2, 8, 6, 1000, 3, 8, 2
+    N = 1 + K + R
+    g = torch.Generator(device=DEV).manual_seed(4)
+    rnd = lambda *s: torch.randn(*s, generator=g, device=DEV).to(torch.bfloat16)
+    L = torch.tensor([70, 300], dtype=torch.int32, device=DEV)
+    caches = 3 if layer_map is None else 2
+    kc, vc = rnd(caches, B, 320, Hkv, 128), rnd(caches, B, 320, Hkv, 128)
+    root = torch.zeros(B, dtype=torch.int32, device=DEV)
+    x = StepInputs(rnd(B, K, V), root, L, None, rnd(layers, B, N, Hq, 128), rnd(layers, B, N, Hkv, 128),
+                   rnd(layers, B, N, Hkv, 128), rnd(B, N, V))
+    gaps = torch.zeros(2 * layers, B, N, Hq, 128, dtype=torch.bfloat16, device=DEV)
+    gaps[::2] = x.q
+    kv = cure.kv_desc(Hkv, 128, 320)
+    results = []
+    for q in (x.q, list(x.q), gaps[::2]):
+        k, v = kc.clone(), vc.clone()
+        st = RepairVerifyStep(B, K, V, 2, 1.0, R, 2, 1, layers, Hq, kv, DEV, layer_map=layer_map)
+        st.attn_out.zero_()
+        r = st.run(StepInputs(x.draft_logits, root, L, None, q, x.tree_k, x.tree_v, x.target_logits), list(k), list(v))
+        assert cure.cure_device_error() == 0
+        # (layers that share a cache write their rows into it in no fixed order)
+        results.append([r["attn"]] + ([k, v] if layer_map is None else []) + [t for part in ("tree", "acc", "resync") for t in r[part].values()])
+    for other in results[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(results[0], other))
+    for l, p in enumerate(layer_map or range(layers)):
+        out = torch.zeros_like(x.q[l])
+        tree = r["tree"]
+        cure.cure_tree_attn(x.q[l], x.tree_k[l], x.tree_v[l], kc[p], vc[p], kv, L, tree["n_nodes"], tree["anc"], st.scale,
+                            out=out)
+        assert torch.equal(out, results[0][0][l])
