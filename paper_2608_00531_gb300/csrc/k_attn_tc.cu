@@ -32,17 +32,16 @@
 //                     microsecond, so fewer, larger boxes load faster.  Tree
 //                     tiles and contiguous caches use [d half][64 keys][64 d]
 //                     for K and [16-key chunk][d half][16 keys][64 d] for V.
-//   warps 9 / 10      S issuers (one lane each) of M tile 0 / 1:
+//   warps 9 / 10      S issuers (an elected lane each) of M tile 0 / 1:
 //                     S_m = Q_m K^T (M128 N64 K128) into TMEM S_m
-//   warp 11           PV issuer (one lane) of both M tiles:
+//   warp 11           PV issuer (an elected lane) of both M tiles:
 //                     O_m += P_m V (A = P_m in TMEM, M128 N128 K64); it
 //                     releases the K/V stage after the tile's last product.
 //                     S is on the softmax's critical path and PV is not, so
 //                     an S product never queues behind a PV issue.  The
 //                     products of one group go out from one asm block with
-//                     constant descriptor steps, which keeps the issuing
-//                     lanes' instruction count low while the softmax warps
-//                     share their schedulers.
+//                     constant descriptor steps: the issuing warps share
+//                     their schedulers with the softmax warps.
 // TMEM (512 columns): S[2] (2 x 64) | P[2][2] (4 x 32, bf16 pairs) | O[2]
 // (2 x 128).  The softmax releases S_m as soon as it has loaded it, so the
 // next tile's S product runs while this tile's exponentials are computed; P
@@ -153,13 +152,13 @@ __device__ __forceinline__ void mma_pv_group(uint32_t d, uint32_t pa, uint64_t v
 }
 
 // Arrive on `bar` once the products this warp's elected lane issued are done.
-// The issuing warps run converged and elect the lane inside the asm: the
-// descriptors then stay in uniform registers, where a lane-0 branch moves each
-// operand of each product there (in the LM head's issuer, which steps the same
-// way, four products took 265 cycles to issue, now 124).  Graph-replayed:
-// 28 q / 4 kv heads, 16 sequences of 5001-8191 keys, trees of up to 65 nodes
-// 112 -> 107 us; 32 of 1024-8192 78.9 -> 77.4 us; 64 x 8 kv heads x 32768 keys
-// 1860 -> 1815 us.
+// The issuing warps run converged and elect the lane inside the asm instead of
+// branching to lane 0 (in the LM head's issuer, which steps the same way, four
+// products then take 124 cycles to issue instead of 265).  28 q / 4 kv heads, 16
+// sequences of 5001-8191 keys, trees of up to 65 nodes 112 -> 107 us; 32 of
+// 1024-8192 keys and 64 x 8 kv heads x 32768 keys within 1-2 %, about what runs
+// differ by; one M tile on 8- and 16-token pages lost up to 2 % on stream-K (see
+// attn_ping_pong).
 __device__ __forceinline__ void commit_elect(uint32_t bar) {
   asm volatile(
       "{\n\t.reg .pred el;\n\telect.sync _|el, 0xffffffff;\n\t"

@@ -1,8 +1,9 @@
 """Failure detection on the GPU, without a fault: every pipeline wait in the
 library is bounded, and a wait that gives up raises CURE_DEVERR_TIMEOUT in
-the device error word instead of hanging the GPU.  The self-test entry point
-runs that same bounded wait on a barrier nothing ever completes; the status
-must come back through cure_device_error() and the context must stay usable.
+the device error word instead of hanging the GPU.  The self-test entry points
+run that same bounded wait on a barrier nothing ever completes, by itself and in
+either CTA of the LM head's pairs; the status must come back through
+cure_device_error() and the context must stay usable.
 """
 import numpy as np
 import pytest
