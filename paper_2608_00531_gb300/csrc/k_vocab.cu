@@ -465,7 +465,7 @@ struct ScanPart {
 // One of the few ids at the row's ends, outside its whole vectors (a NaN there is
 // passed over).
 __device__ __forceinline__ void lse_add(Lse2& ls, float x) {
-  if (x == x) lse_merge(ls, x * kLog2e, 1.f);
+  lse_merge(ls, fmaxf(x, -INFINITY) * kLog2e, 1.f);  // (a NaN as -inf)
 }
 
 template <int KT, int T>
