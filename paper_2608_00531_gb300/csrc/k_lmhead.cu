@@ -371,15 +371,17 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap mh, const __grid_const
           st_cluster(base + 8 * BN * 4 + (c * 32 + lane) * 4, (uint32_t)bi[j]);
         }
       }
+    } else if (lane == 0) {
+      // the pair gives up together: with a wait run out in either CTA (whatever its
+      // role, that CTA's epilogue stops) the ring need not hold maxima, and the
+      // range reports none, so that no stale word becomes a token
+      st_cluster(in_first_cta(sb + kOffAbort), 1u);
     }
   }
 
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  // the pair gives up together: with a wait run out in either CTA the ring need not
-  // hold maxima, and the range reports none, so that no stale word becomes a token
-  if (threadIdx.x == 0 && *abort_flag) st_cluster(in_first_cta(sb + kOffAbort), 1u);
   cluster_sync();
   if (rank == 0 && (int)threadIdx.x < A.nt && n0 + (int)threadIdx.x < A.M) {
     const bool whole = !*abort_flag;
